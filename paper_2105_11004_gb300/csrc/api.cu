@@ -527,7 +527,7 @@ int select_common(lev_handle* h, const float* Atilde, int64_t m, int64_t d, cons
     if (k >= d) return LEV_OK;
     LEV_TRY(ensure(h->omega_rs, sizeof(double) * (size_t)d * d));
     double* Rs = (double*)h->omega_rs.ptr;
-    LEV_CUDA(lev::launch_gram_fp64(Atilde, d, m, d, qs->Gp, qs->G, st));
+    LEV_CUDA(lev::launch_gram_fp64(Atilde, d, m, d, qs->Gp, qs->G, h->status, st));
     const int64_t max_swaps = 64 * d;
     double* host_out = reinterpret_cast<double*>(h->host_rank + 2);
     for (int64_t it = 0;; ++it) {
@@ -586,7 +586,7 @@ int csr_gram(lev_handle* h, const int64_t* row_ptr, const int32_t* col, const fl
         double* Gp2 = Gh + (size_t)d * d;
         float* H = reinterpret_cast<float*>(Gp2 + gp);
         LEV_CUDA(lev::launch_densify_rows(row_ptr, col, val, hidx, hcount, nh, d, H, st));
-        LEV_CUDA(lev::launch_gram_fp64(H, d, nh, d, Gp2, Gh, st));
+        LEV_CUDA(lev::launch_gram_fp64(H, d, nh, d, Gp2, Gh, h->status, st));
         Gheavy = Gh;
     }
     LEV_CUDA(lev::launch_gram_csr_light(row_ptr, col, val, n, d, max_len, Gheavy, G, st));
@@ -599,7 +599,7 @@ int final_csr(lev_handle* h, const int64_t* rp, const int32_t* cl, const float* 
               const float* Mfull, int64_t k, float* theta, cudaStream_t st) {
     if (lev::csr_gram_pays(n, d, nnz, k)) {
         LEV_TRY(ensure(h->csr_p, lev::csr_gram_scratch_bytes(d, k)));
-        LEV_CUDA(lev::launch_final_csr_gram(rp, cl, vl, n, d, Mfull, k, h->csr_p.ptr, theta, st));
+        LEV_CUDA(lev::launch_final_csr_gram(rp, cl, vl, n, d, Mfull, k, h->csr_p.ptr, theta, h->status, st));
         return LEV_OK;
     }
     LEV_CUDA(lev::launch_final_csr_fp32(rp, cl, vl, n, d, Mfull, k, theta, st));
@@ -1073,7 +1073,7 @@ int lev_exact_dense(lev_handle* h, const float* A, int64_t n, int64_t d, int64_t
     LEV_TRY(ensure(h->exact_gp, sizeof(double) * lev::gram_partial_doubles(n, d)));
     lev::QrScratch q2 = qs;
     q2.Gp = (double*)h->exact_gp.ptr;
-    LEV_CUDA(lev::launch_gram_fp64(A, lda, n, d, q2.Gp, q2.G, st));
+    LEV_CUDA(lev::launch_gram_fp64(A, lda, n, d, q2.Gp, q2.G, h->status, st));
     LEV_CUDA(lev::launch_factor_gram(n, d, tau_of(p), perm, k, q2, perm, (double*)h->R.ptr, h->status, st));
     int64_t k2 = 0;
     rc = finish(h, q2, &k2, st);
@@ -1196,7 +1196,7 @@ int lev_exact_reference_dense(lev_handle* h, const float* A, int64_t n, int64_t 
     lev::qr_scratch_carve(h->qr.ptr, 1, d, &q);
     LEV_TRY(ensure(h->exact_gp, sizeof(double) * lev::gram_partial_doubles(n, d)));
     q.Gp = (double*)h->exact_gp.ptr;
-    LEV_CUDA(lev::launch_gram_fp64(A, lda, n, d, q.Gp, q.G, st));
+    LEV_CUDA(lev::launch_gram_fp64(A, lda, n, d, q.Gp, q.G, h->status, st));
     return exact_reference_tail(h, q, n, d, tau, A, lda, nullptr, nullptr, nullptr, 0, theta, rank, perm, st);
 }
 

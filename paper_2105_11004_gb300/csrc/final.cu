@@ -388,7 +388,8 @@ bool csr_gram_pays(int64_t n, int64_t d, int64_t nnz, int64_t k) {
 }
 
 cudaError_t launch_final_csr_gram(const int64_t* row_ptr, const int32_t* col, const float* val, int64_t n, int64_t d,
-                                  const float* Mfull, int64_t k, void* scratch, float* theta, cudaStream_t st) {
+                                  const float* Mfull, int64_t k, void* scratch, float* theta, int32_t* status,
+                                 cudaStream_t st) {
     double* P = reinterpret_cast<double*>(scratch);
     double* Gp = P + d * d;
     float* MT = reinterpret_cast<float*>(Gp + gram_partial_doubles(k, d));
@@ -396,7 +397,7 @@ cudaError_t launch_final_csr_gram(const int64_t* row_ptr, const int32_t* col, co
     int tg = (int)((d * k + 255) / 256);
     if (tg > 152 * 8) tg = 152 * 8;
     k_transpose_mfull<<<tg, 256, 0, st>>>(Mfull, (int)d, (int)k, MT);
-    cudaError_t e = launch_gram_fp64(MT, d, k, d, Gp, P, st);           // P = Mfull Mfull^T (FP64-grade)
+    cudaError_t e = launch_gram_fp64(MT, d, k, d, Gp, P, status, st);           // P = Mfull Mfull^T (FP64-grade)
     if (e != cudaSuccess) return e;
     k_split_pairs<<<152 * 4, 256, 0, st>>>(P, d * d, Pdf);
     const bool vec = (reinterpret_cast<uintptr_t>(Mfull) % 16 == 0) && (k % 4 == 0);

@@ -19,7 +19,8 @@
 //     FP64 sum over blocks, comparable to the m u_64 sum |a b| of an FP64 FMA
 //     chain at the sketch sizes (m = 1,024 to 4,096).
 //     Upper 32 x 32 tiles split over rows, split partials reduced in a fixed
-//     order and mirrored;
+//     order and mirrored. From 1.5e8 products on the tensor-core kernel of
+//     gram_tc.cu takes its place (1.03 -> 0.18 ms at 4096 x 1024);
 //   k_pchol_grid: one cooperative grid (at most one CTA per SM; ceil(d/3) CTAs
 //     up to d = 256, where a step is latency-bound; above d = 256 one thread a
 //     row, 512 or 1,024 threads a CTA); CTA c owns the
@@ -776,10 +777,10 @@ __global__ void k_df_to_fp64(double* __restrict__ R, const double* __restrict__ 
 
 }  // namespace
 
-// Row splits of the Gram product. The FP64 pipe of an SM is shared by its resident CTAs, so the
+// Row splits of the compensated Gram product. The FP64 pipe of an SM is shared by its resident CTAs, so the
 // SM with the most CTAs sets the time: take the split count whose CTA total fills its last wave
 // over the SMs best (the largest such count within 1%), with the FP64 partials held to 4 MB.
-int gram_splits(int64_t m, int64_t d) {
+static int gram_splits(int64_t m, int64_t d) {
     static std::atomic<int> sms_cached{0};               // host threads share it
     int sms = sms_cached.load(std::memory_order_relaxed);
     if (sms == 0) {
@@ -807,12 +808,22 @@ int gram_splits(int64_t m, int64_t d) {
     return (int)best;
 }
 
-size_t gram_partial_doubles(int64_t m, int64_t d) {
+static size_t dot2_partial_doubles(int64_t m, int64_t d) {
     return (size_t)gram_splits(m, d) * gram_tiles((int)d) * GT * GT;
 }
 
+// The tensor-core kernel (gram_tc.cu) from 1.5e8 products on: it takes 40 to 60 us whatever the shape, the
+// compensated kernel about that at 1.5e8. Below 33 columns most of a 128-column tile is padding. No shape that
+// fits lev_rrqr_noalloc's 8 MiB has so many products, so its working set is the compensated kernel's.
+static bool gram_tc_pays(int64_t m, int64_t d) { return d > 32 && (double)m * (double)d * (double)(d + 32) >= 3.0e8; }
+
+size_t gram_partial_doubles(int64_t m, int64_t d) {
+    return gram_tc_pays(m, d) ? gram_tc_partial_doubles(m, d) : dot2_partial_doubles(m, d);
+}
+
 cudaError_t launch_gram_fp64(const float* A, int64_t lda, int64_t m, int64_t d, double* Gp, double* G,
-                             cudaStream_t st) {
+                             int32_t* status, cudaStream_t st) {
+    if (gram_tc_pays(m, d)) return launch_gram_tc(A, lda, m, d, Gp, G, status, st);
     const int splits = gram_splits(m, d);
     const int rows_per_split = (int)(((m + splits - 1) / splits + kDot2Rows - 1) / kDot2Rows * kDot2Rows);
     dim3 grid((unsigned)gram_tiles((int)d), (unsigned)splits);
@@ -866,7 +877,7 @@ cudaError_t launch_densify_rows(const int64_t* row_ptr, const int32_t* col, cons
 cudaError_t launch_gram_pivoted_cholesky(const float* Atilde, int64_t m, int64_t d, double tau,
                                          const int32_t* forced, int64_t forced_rank, const QrScratch& q,
                                          int32_t* status, cudaStream_t st, cudaEvent_t after_gram) {
-    cudaError_t e = launch_gram_fp64(Atilde, d, m, d, q.Gp, q.G, st);
+    cudaError_t e = launch_gram_fp64(Atilde, d, m, d, q.Gp, q.G, status, st);
     if (e != cudaSuccess) return e;
     if (after_gram && (e = cudaEventRecord(after_gram, st)) != cudaSuccess) return e;
     return launch_pivoted_cholesky(m, d, tau, forced, forced_rank, q, status, st);

@@ -81,12 +81,15 @@ cudaError_t launch_segment_sort(const int* off, int64_t s, const uint32_t* in, u
 
 // Gram route of the pivoted QR (gramqr.cu): G = A~^T A~ in FP64, then a
 // pivoted Cholesky on one cooperative grid; fills Rorig, piv and rank.
-int gram_splits(int64_t m, int64_t d);
 size_t gram_partial_doubles(int64_t m, int64_t d);
 // G (d x d FP64, both triangles) = A^T A for A (m x d FP32, leading dimension lda); Gp holds
-// gram_partial_doubles(m, d) doubles of split partials.
+// gram_partial_doubles(m, d) doubles of split partials. status: device status word.
 cudaError_t launch_gram_fp64(const float* A, int64_t lda, int64_t m, int64_t d, double* Gp, double* G,
-                             cudaStream_t st);
+                             int32_t* status, cudaStream_t st);
+// The tensor-core form (gram_tc.cu).
+size_t gram_tc_partial_doubles(int64_t m, int64_t d);
+cudaError_t launch_gram_tc(const float* A, int64_t lda, int64_t m, int64_t d, double* Gp, double* G, int32_t* status,
+                           cudaStream_t st);
 // G (d x d FP64, both triangles) = A^T A for CSR A (n rows) by the rows' outer products, FP64
 // atomics (the order of the sums varies between runs).
 cudaError_t launch_gram_csr_fp64(const int64_t* row_ptr, const int32_t* col, const float* val, int64_t n,
@@ -198,7 +201,8 @@ cudaError_t launch_final_dense_fp32(const float* A, int64_t lda, int64_t n, int6
 size_t csr_gram_scratch_bytes(int64_t d, int64_t k);
 bool csr_gram_pays(int64_t n, int64_t d, int64_t nnz, int64_t k);
 cudaError_t launch_final_csr_gram(const int64_t* row_ptr, const int32_t* col, const float* val, int64_t n, int64_t d,
-                                  const float* Mfull, int64_t k, void* scratch, float* theta, cudaStream_t st);
+                                  const float* Mfull, int64_t k, void* scratch, float* theta, int32_t* status,
+                                  cudaStream_t st);
 cudaError_t launch_final_csr_fp32(const int64_t* row_ptr, const int32_t* col, const float* val,
                                   int64_t n, int64_t d, const float* Mfull, int64_t k,
                                   float* theta, cudaStream_t st);
