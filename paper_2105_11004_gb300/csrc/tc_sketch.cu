@@ -249,19 +249,20 @@ __global__ void __launch_bounds__(192, 1) k_gauss_tc(const __grid_constant__ CUt
                 uint32_t r[32];
                 tmem_ld32(tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)c0, r);
                 tmem_ld_wait();
-                const int col0 = ntile * nt + c0;
-                if (row >= m) continue;
-                if (vec && col0 + 32 <= d) {
+                // the tile ends at column nt: the accumulator columns past it are not this tile's
+                const int col0 = ntile * nt + c0, ce = min(min(32, nt - c0), d - col0);
+                if (row < m && vec && ce == 32) {
 #pragma unroll
                     for (int j = 0; j < 32; j += 4)
                         *reinterpret_cast<float4*>(out + col0 + j) =
                             make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]),
                                         __uint_as_float(r[j + 3]));
-                } else {
+                } else if (row < m) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
-                        if (col0 + j < d) out[col0 + j] = __uint_as_float(r[j]);
+                        if (j < ce) out[col0 + j] = __uint_as_float(r[j]);
                 }
+                __syncwarp();                              // the next tcgen05.ld is the whole warp's
             }
         }
     }
