@@ -44,6 +44,7 @@
 
 #include <algorithm>
 
+#include "f32x2.cuh"
 #include "lev_common.cuh"
 #include "lev_kernels.cuh"
 #include "tc_common.cuh"
@@ -114,33 +115,6 @@ __device__ __forceinline__ int column_exponent(uint32_t maxbits) {
     return e < -119 ? -119 : e;
 }
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
-
-// Two FP32 numbers in one 64-bit register, added with one instruction each (round to nearest, no
-// contraction): the converters and the fetchers are bound by issue slots.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 
 __device__ __forceinline__ void store_digit(uint8_t* dst, const f32x2 (&t)[4]) {
     uint4 v;

@@ -3,14 +3,18 @@
 //  * singular values of the sketch: one-sided (Hestenes) Jacobi on the rows of R, the triangular
 //    factor of A~ P (sigma(R) = sigma(A~)): plane rotations of row pairs (Y <- J Y) until every
 //    pair is orthogonal, after which the row norms are the singular values and the normalised rows
-//    the right singular vectors of R. One cooperative grid; the pairs of a round are disjoint
-//    (round-robin order), a bounded grid barrier separates the rounds. The rank is then the count
+//    the right singular vectors of R. One thread-block cluster with the rows in shared memory up to
+//    d = 384, one cooperative grid above (the pairs of a round are disjoint, round-robin order). The rank is then the count
 //    of sigma_j > tau sigma_1 (Alg. 11 step 3; Sec. 7.2: the singular values see a gap that the
 //    diagonal of R can miss);
 //  * strong-RRQR measures at a fixed k (Alg. 2 after Gu and Eisenstat): from R in pivot order,
 //    Z = R11^{-1} [I | R12], the row norms of R11^{-1}, gamma_j^2 = G_jj - ||R[:k, j]||^2 (the
 //    Schur complement's diagonal, G = A~^T A~), and the largest
 //    rho_ij^2 = (R11^{-1} R12)_ij^2 + gamma_j^2 ||e_i^T R11^{-1}||^2 with its (i, j).
+#include <atomic>
+
+#include "df.cuh"
+#include "f32x2.cuh"
 #include "lev_common.cuh"
 #include "lev_kernels.cuh"
 
@@ -236,6 +240,330 @@ __global__ void __launch_bounds__(256) k_jacobi_rows(float* __restrict__ Yh, flo
     if (blockIdx.x == 0 && tid == 0) *sweeps_out = max_sweeps + 1;
 }
 
+// ---- the same Jacobi on one thread-block cluster, the rows in shared memory (d up to about 400) ----
+// k_jacobi_rows spends a round on L2: two row versions polled, two rows read, written and released, about
+// 7.5 us for one pair a CTA, whatever the arithmetic. Here the r rows are cut into 2 C blocks of b rows, two
+// blocks a CTA (C = 1 .. 16 CTAs, b = 8 at d = 256), and a sweep is 2 C - 1 block rounds of the round-robin
+// tournament: a CTA takes the b x b pairs between its two blocks in b steps of b disjoint pairs, a warp a
+// pair, and the blocks then move on through distributed shared memory (each CTA pulls its next two blocks
+// into its other buffer; one cluster barrier a block round). The pairs inside the blocks come first. A warp
+// keeps its row of the first block in registers through the b steps. The squared row norms are carried
+// (recomputed every sweep), so a pair costs one dot product; the rotation's tangent is taken in FP32 (its
+// error of 1e-7 leaves 1e-7 of the pair's dot product to the next sweep) and made a rotation in double-float,
+// c = 1 / sqrt(1 + t^2), s = c t, which is what keeps the rows' accuracy. Two elements an instruction
+// (packed FP32). Same stopping rule as k_jacobi_rows; singular values at d = 256: 5.7e-14 off (8.8e-14 there).
+// The SVD path with its QR: 24.1 -> 6.5 ms at 1,024 x 256 (Jacobi 21.5 -> 3.4), 7.9 -> 1.8 at d = 99, 45.4 -> 15.6
+// at d = 384. A pair is a chain of about 2,500 cycles: dot product and its warp sum, rotation, update, barrier.
+// A row held by a warp: lane l has elements 128 q + 4 l .. + 3, as 2 Q packed pairs of high and low parts.
+template <int Q>
+struct JRow {
+    f32x2 h[2 * Q], l[2 * Q];
+};
+template <int Q>
+__device__ __forceinline__ void load_row(const float* row, int dp, int lane, JRow<Q>& v) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(row + 128 * q + 4 * lane);
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(row + dp + 128 * q + 4 * lane);
+        v.h[2 * q] = a.x; v.h[2 * q + 1] = a.y;
+        v.l[2 * q] = b.x; v.l[2 * q + 1] = b.y;
+    }
+}
+template <int Q>
+__device__ __forceinline__ void store_row(float* row, int dp, int lane, const JRow<Q>& v) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        *reinterpret_cast<ulonglong2*>(row + 128 * q + 4 * lane) = make_ulonglong2(v.h[2 * q], v.h[2 * q + 1]);
+        *reinterpret_cast<ulonglong2*>(row + dp + 128 * q + 4 * lane) = make_ulonglong2(v.l[2 * q], v.l[2 * q + 1]);
+    }
+}
+// x . y over the warp (the same pair on every lane): compensated as df_dot_acc, two elements at a time
+template <int Q>
+__device__ __forceinline__ float2 row_dot(const JRow<Q>& x, const JRow<Q>& y) {
+    f32x2 s = 0ull, c = 0ull;
+#pragma unroll
+    for (int k = 0; k < 2 * Q; ++k) {
+        const f32x2 p = mul2(x.h[k], y.h[k]);
+        f32x2 e = fma2(x.h[k], y.h[k], neg2(p));
+        e = fma2(x.h[k], y.l[k], e);
+        e = fma2(x.l[k], y.h[k], e);
+        const f32x2 s1 = add2(s, p), z = sub2(s1, s);
+        c = add2(c, add2(add2(sub2(s, sub2(s1, z)), sub2(p, z)), e));
+        s = s1;
+    }
+    float s0, s1, c0, c1, h, l;
+    unpack2(s, s0, s1);
+    unpack2(c, c0, c1);
+    df_add(s0, c0, s1, c1, h, l);
+    df_warp_sum(h, l);
+    return make_float2(h, l);
+}
+// (ah + al) u + (bh + bl) v for packed double-float u, v and scalars broadcast to both halves
+__device__ __forceinline__ void df_axpby(f32x2 ah, f32x2 al, f32x2 uh, f32x2 ul, f32x2 bh, f32x2 bl, f32x2 vh, f32x2 vl,
+                                         f32x2& oh, f32x2& ol) {
+    const f32x2 p = mul2(ah, uh), q = mul2(bh, vh);
+    f32x2 e = fma2(ah, uh, neg2(p)), f = fma2(bh, vh, neg2(q));
+    e = fma2(ah, ul, e);
+    f = fma2(bh, vl, f);
+    e = fma2(al, uh, e);
+    f = fma2(bl, vh, f);
+    const f32x2 s = add2(p, q), z = sub2(s, p);
+    f32x2 r = add2(sub2(p, sub2(s, z)), sub2(q, z));
+    r = add2(r, add2(e, f));
+    oh = add2(s, r);
+    ol = sub2(r, sub2(oh, s));
+}
+// 1 / sqrt(v) for v = vh + vl in [1, 2]: an FP32 estimate y with residual e = 1 - v y^2 (about 2^-23; its leading
+// difference is exact), then y (1 + e / 2 + 3 e^2 / 8).
+__device__ __forceinline__ float2 inv_sqrt_1to2(float vh, float vl) {
+    float y = rsqrtf(vh);
+    y = __fmul_rn(y, __fmaf_rn(__fmul_rn(-0.5f, vh), __fmul_rn(y, y), 1.5f));
+    const float yy = __fmul_rn(y, y), yye = __fmaf_rn(y, y, -yy);
+    const float p = __fmul_rn(vh, yy), pe = __fmaf_rn(vh, yy, -p);
+    const float e = __fsub_rn(__fsub_rn(1.f, p), __fadd_rn(pe, __fmaf_rn(vh, yye, __fmul_rn(vl, yy))));
+    const float corr = __fmul_rn(y, __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f)));
+    const float h = __fadd_rn(y, corr);
+    return make_float2(h, __fsub_rn(corr, __fsub_rn(h, y)));
+}
+// The pair (cs, sn) made orthonormal to a few 2^-50: the residual 1 - cs^2 - sn^2 (its leading differences are
+// exact, the other terms summed error-free) goes half into each low part. An error here scales both rows at
+// every rotation; the FP64 rotations of k_jacobi_rows, split into pairs, have the same 8e-16.
+__device__ __forceinline__ void orthonormalise(float2& cs, float2& sn) {
+    const float p1 = __fmul_rn(cs.x, cs.x), e1 = __fmaf_rn(cs.x, cs.x, -p1);
+    const float p2 = __fmul_rn(sn.x, sn.x), e2 = __fmaf_rn(sn.x, sn.x, -p2);
+    const float c2 = 2.f * cs.x, s2 = 2.f * sn.x;
+    const float m1 = __fmul_rn(c2, cs.y), n1 = __fmaf_rn(c2, cs.y, -m1);
+    const float m2 = __fmul_rn(s2, sn.y), n2 = __fmaf_rn(s2, sn.y, -m2);
+    float s = __fsub_rn(__fsub_rn(1.f, p1), p2), a, b, c, d;
+    two_sum(s, -e1, s, a);
+    two_sum(s, -e2, s, b);
+    two_sum(s, -m1, s, c);
+    two_sum(s, -m2, s, d);
+    const float low = __fsub_rn(__fadd_rn(__fadd_rn(a, b), __fadd_rn(c, d)),
+                                __fadd_rn(__fadd_rn(n1, n2), __fmaf_rn(cs.y, cs.y, __fmul_rn(sn.y, sn.y))));
+    const float half = 0.5f * __fadd_rn(s, low);
+    cs.y = __fmaf_rn(cs.x, half, cs.y);
+    sn.y = __fmaf_rn(sn.x, half, sn.y);
+}
+// Rotate rows x, y (squared norms a, b) so that they become orthogonal; false if they count as orthogonal.
+template <int Q>
+__device__ __forceinline__ bool rotate_rows(JRow<Q>& x, JRow<Q>& y, float2& a, float2& b) {
+    const float2 c = row_dot<Q>(x, y);
+    if (!(a.x > 0.f && b.x > 0.f && fabsf(c.x) > (float)kJacobiTol * sqrtf(a.x) * sqrtf(b.x))) return false;
+    const float zeta = ((b.x - a.x) + (b.y - a.y)) / (2.f * c.x);
+    const float az = fabsf(zeta);
+    const float t = copysignf(az > 1e9f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(az, az, 1.f))), zeta);
+    const float tt = __fmul_rn(t, t), tte = __fmaf_rn(t, t, -tt);
+    const float vh = __fadd_rn(1.f, tt);
+    const float vl = __fadd_rn(__fsub_rn(tt, __fsub_rn(vh, 1.f)), tte);                 // 1 + t^2 (t^2 <= 1)
+    float2 cs = inv_sqrt_1to2(vh, vl), sn = lev::df_mul(cs, make_float2(t, 0.f));
+    orthonormalise(cs, sn);
+    const f32x2 ch = pack2(cs.x, cs.x), cl = pack2(cs.y, cs.y), sh = pack2(sn.x, sn.x), sl = pack2(sn.y, sn.y);
+    const f32x2 nsh = pack2(-sn.x, -sn.x), nsl = pack2(-sn.y, -sn.y);
+#pragma unroll
+    for (int k = 0; k < 2 * Q; ++k) {
+        f32x2 xh, xl;
+        df_axpby(ch, cl, x.h[k], x.l[k], nsh, nsl, y.h[k], y.l[k], xh, xl);             // x' = cs x - sn y
+        df_axpby(sh, sl, x.h[k], x.l[k], ch, cl, y.h[k], y.l[k], y.h[k], y.l[k]);       // y' = sn x + cs y
+        x.h[k] = xh;
+        x.l[k] = xl;
+    }
+    const float2 tc = lev::df_mul(c, make_float2(t, 0.f));
+    float h, l;
+    df_add(a.x, a.y, -tc.x, -tc.y, h, l);
+    a = make_float2(h, l);
+    df_add(b.x, b.y, tc.x, tc.y, h, l);
+    b = make_float2(h, l);
+    return true;
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t remote_addr(const void* p, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ uint4 remote_ld16(uint32_t a) {
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+    return v;
+}
+
+constexpr int kJacobiMaxWarps = 16;
+
+// bmax: rows a block holds at most (warps of the CTA); dp = 128 Q >= d. Dynamic shared memory: two buffers of
+// two blocks of bmax rows of 2 dp floats (high parts, low parts).
+template <int Q>
+__global__ void __launch_bounds__(32 * kJacobiMaxWarps, 1) k_jacobi_cluster(float* __restrict__ Yh, float* __restrict__ Yl,
+                                                                           const int64_t* __restrict__ d_rows, int d,
+                                                                           int bmax, int max_sweeps,
+                                                                           int32_t* __restrict__ sweeps_out) {
+    constexpr int dp = 128 * Q;
+    extern __shared__ __align__(16) float jrows[];
+    __shared__ __align__(16) float2 norm_s[2][2][kJacobiMaxWarps];   // by buffer and block: squared norms
+    __shared__ __align__(16) int id_s[2][2][kJacobiMaxWarps];        // rows of Y held (-1: none)
+    __shared__ int rotated_s[2];
+    uint32_t C, me;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(me));
+    const int r = (int)min(max(*d_rows, (int64_t)0), (int64_t)d);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int b = (r + 2 * (int)C - 1) / (2 * (int)C);
+    if (r < 2) {                                            // the same in every CTA
+        if (me == 0 && threadIdx.x == 0) *sweeps_out = 0;
+        return;
+    }
+    auto row = [&](int buf, int blk, int i) -> float* { return jrows + ((size_t)(buf * 2 + blk) * bmax + i) * (2 * dp); };
+    // blocks 2 me and 2 me + 1
+    for (int blk = 0; blk < 2; ++blk)
+        for (int i = w; i < b; i += nw) {
+            const int id = (2 * (int)me + blk) * b + i;
+            float* dst = row(0, blk, i);
+            for (int e = lane; e < dp; e += 32) {
+                const bool ok = id < r && e < d;
+                dst[e] = ok ? Yh[(int64_t)id * d + e] : 0.f;
+                dst[dp + e] = ok ? Yl[(int64_t)id * d + e] : 0.f;
+            }
+            if (lane == 0) id_s[0][blk][i] = id < r ? id : -1;
+        }
+    if (threadIdx.x < 2) rotated_s[threadIdx.x] = 0;
+    __syncthreads();
+    int buf = 0, sweep = 0;
+    const int rounds = 2 * (int)C - 1;
+    for (; sweep < max_sweeps; ++sweep) {
+        int rotations = 0;                                 // by this warp (lane 0's count)
+        // squared norms afresh
+        for (int i = w; i < 2 * b; i += nw) {
+            JRow<Q> x;
+            load_row<Q>(row(buf, i / b, i % b), dp, lane, x);
+            const float2 n2 = row_dot<Q>(x, x);
+            if (lane == 0) norm_s[buf][i / b][i % b] = n2;
+        }
+        __syncthreads();
+        // the pairs inside the two blocks
+        const int n = b + (b & 1);
+        for (int t = 0; t < n - 1; ++t) {
+            for (int e = w; e < n; e += nw) {                // n / 2 pairs a block
+                const int blk = e / (n / 2);
+                int p, q;
+                round_pair(n, t, e % (n / 2), p, q);
+                if (p >= b || q >= b || id_s[buf][blk][p] < 0 || id_s[buf][blk][q] < 0) continue;
+                if (p > q) { const int x = p; p = q; q = x; }
+                JRow<Q> x, y;
+                load_row<Q>(row(buf, blk, p), dp, lane, x);
+                load_row<Q>(row(buf, blk, q), dp, lane, y);
+                float2 na = norm_s[buf][blk][p], nb = norm_s[buf][blk][q];
+                if (rotate_rows<Q>(x, y, na, nb)) {
+                    store_row<Q>(row(buf, blk, p), dp, lane, x);
+                    store_row<Q>(row(buf, blk, q), dp, lane, y);
+                    if (lane == 0) { norm_s[buf][blk][p] = na; norm_s[buf][blk][q] = nb; }
+                    ++rotations;
+                }
+            }
+            __syncthreads();
+        }
+        for (int rd = 0; rd < rounds; ++rd) {
+            // warp w holds row w of the first block; step k pairs it with row (w + k) mod b of the second
+            const bool mine = w < b && id_s[buf][0][w] >= 0;
+            JRow<Q> x;
+            float2 na = make_float2(0.f, 0.f);
+            bool changed = false;
+            if (mine) {
+                load_row<Q>(row(buf, 0, w), dp, lane, x);
+                na = norm_s[buf][0][w];
+            }
+            for (int k = 0; k < b; ++k) {
+                if (mine) {
+                    const int j = w + k < b ? w + k : w + k - b;
+                    if (id_s[buf][1][j] >= 0) {
+                        JRow<Q> y;
+                        load_row<Q>(row(buf, 1, j), dp, lane, y);
+                        float2 nb = norm_s[buf][1][j];
+                        if (rotate_rows<Q>(x, y, na, nb)) {
+                            store_row<Q>(row(buf, 1, j), dp, lane, y);
+                            if (lane == 0) norm_s[buf][1][j] = nb;
+                            changed = true;
+                            ++rotations;
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+            if (changed) {
+                store_row<Q>(row(buf, 0, w), dp, lane, x);
+                if (lane == 0) norm_s[buf][0][w] = na;
+            }
+            if (rd == rounds - 1 && lane == 0 && rotations) atomicAdd(&rotated_s[sweep & 1], rotations);
+            if (C == 1) {
+                __syncthreads();
+                break;
+            }
+            // the tournament's next blocks: first <- first of CTA me - 1 (CTA 1: second of CTA 0; CTA 0 keeps
+            // its own), second <- second of CTA me + 1 (the last CTA: its own first)
+            cluster_barrier();
+            const int nb2 = buf ^ 1;
+            for (int blk = 0; blk < 2; ++blk) {
+                int from, fb;
+                if (blk == 0) {
+                    from = me == 0 ? 0 : (int)me - 1;
+                    fb = me == 1 ? 1 : 0;
+                } else {
+                    from = me + 1 < C ? (int)me + 1 : (int)me;
+                    fb = me + 1 < C ? 1 : 0;
+                }
+                const uint32_t src = remote_addr(row(buf, fb, 0), from);
+                uint4* dst = reinterpret_cast<uint4*>(row(nb2, blk, 0));
+                const int count = b * 2 * dp / 4;
+                for (int e = threadIdx.x; e < count; e += 4 * blockDim.x) {
+                    uint4 v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (e + u * (int)blockDim.x < count) v[u] = remote_ld16(src + 16u * (uint32_t)(e + u * blockDim.x));
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (e + u * (int)blockDim.x < count) dst[e + u * blockDim.x] = v[u];
+                }
+                if (threadIdx.x < kJacobiMaxWarps / 2)
+                    reinterpret_cast<uint4*>(norm_s[nb2][blk])[threadIdx.x] =
+                        remote_ld16(remote_addr(norm_s[buf][fb], from) + 16u * threadIdx.x);
+                else if (threadIdx.x < kJacobiMaxWarps / 2 + kJacobiMaxWarps / 4)
+                    reinterpret_cast<uint4*>(id_s[nb2][blk])[threadIdx.x - kJacobiMaxWarps / 2] =
+                        remote_ld16(remote_addr(id_s[buf][fb], from) + 16u * (threadIdx.x - kJacobiMaxWarps / 2));
+            }
+            buf = nb2;
+            __syncthreads();
+        }
+        // rotations of the sweep in every CTA (two counters, the other one cleared for the next sweep)
+        int total = rotated_s[sweep & 1];
+        if (C > 1) {
+            total = 0;
+            for (uint32_t c = 0; c < C; ++c) {
+                uint32_t v;
+                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(remote_addr(&rotated_s[sweep & 1], (int)c)) : "memory");
+                total += (int)v;
+            }
+        }
+        if (total == 0) break;
+        __syncthreads();
+        if (threadIdx.x == 0) rotated_s[(sweep + 1) & 1] = 0;
+        __syncthreads();
+    }
+    if (me == 0 && threadIdx.x == 0) *sweeps_out = sweep < max_sweeps ? sweep + 1 : max_sweeps + 1;
+    for (int blk = 0; blk < 2; ++blk)
+        for (int i = w; i < b; i += nw) {
+            const int id = id_s[buf][blk][i];
+            if (id < 0) continue;
+            const float* src = row(buf, blk, i);
+            for (int e = lane; e < d; e += 32) {
+                Yh[(int64_t)id * d + e] = src[e];
+                Yl[(int64_t)id * d + e] = src[dp + e];
+            }
+        }
+    if (C > 1) cluster_barrier();                          // no CTA leaves while another may read its shared memory
+}
+
 // sigma (d, descending; zeros past the r rows) and order (the row of Y that holds each) from the
 // row norms of Y; *rank_out = #{sigma_j > tau sigma_1}. One CTA of 1024 threads, bitonic sort of
 // (sigma, row) pairs, ties to the lower row.
@@ -411,6 +739,54 @@ __global__ void k_srrqr_swap(const double* __restrict__ out, double phi2, int32_
 // of the Jacobi (d uint32, from the sweep count + 2), and the double-float rows (2 d^2 FP32).
 size_t rank_scratch_doubles(int64_t d) { return (size_t)(d * d + 3 * d + 16 + 2 * 1024 + 32 + d + 8 + d + d * d + 8); }
 
+// The cluster form: C CTAs, bmax rows a block. cudaErrorNotSupported (nothing launched) where the rows do not
+// fit or no such cluster can be resident.
+template <int Q>
+static cudaError_t launch_jacobi_cluster(float* Yh, float* Yl, const int64_t* d_rows, int d, int C, int max_sweeps,
+                                         int32_t* sweeps_out, cudaStream_t st) {
+    static std::atomic<int> resident[2][64] = {};           // per (C > 8, device): 1 yes, -1 no, 0 unknown
+    const int bmax = (d + 2 * C - 1) / (2 * C);
+    const size_t smem = sizeof(float) * 2 * 2 * (size_t)bmax * 2 * 128 * Q;
+    if (bmax > kJacobiMaxWarps || smem > 220 * 1024) return cudaErrorNotSupported;
+    cudaError_t e;
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    std::atomic<int>* known = dev >= 0 && dev < 64 ? &resident[C > 8 ? 1 : 0][dev] : nullptr;
+    if (known && known->load(std::memory_order_relaxed) < 0) return cudaErrorNotSupported;
+    if ((e = cudaFuncSetAttribute(k_jacobi_cluster<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024)) != cudaSuccess)
+        return e;
+    if (C > 8 && cudaFuncSetAttribute(k_jacobi_cluster<Q>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return cudaErrorNotSupported;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)C);
+    cfg.blockDim = dim3(32u * (unsigned)bmax);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (!known || known->load(std::memory_order_relaxed) == 0) {
+        cudaLaunchConfig_t big = cfg;                        // the largest footprint of this instance
+        big.blockDim = dim3(32 * kJacobiMaxWarps);
+        big.dynamicSmemBytes = 220 * 1024;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, k_jacobi_cluster<Q>, &big) != cudaSuccess || clusters < 1) {
+            cudaGetLastError();
+            if (known) known->store(-1, std::memory_order_relaxed);
+            return cudaErrorNotSupported;
+        }
+        if (known) known->store(1, std::memory_order_relaxed);
+    }
+    e = cudaLaunchKernelEx(&cfg, k_jacobi_cluster<Q>, Yh, Yl, d_rows, d, bmax, max_sweeps, sweeps_out);
+    return e;
+}
+
 cudaError_t launch_svd_rank(const double* R, const int64_t* d_rows, int64_t d, double tau, double* Y, float* Yhl,
                             unsigned* work, double* sigma, int32_t* order, int64_t* rank_out, int32_t* sweeps_out,
                             unsigned* version, int32_t* status, int num_sms, cudaStream_t st) {
@@ -422,21 +798,30 @@ cudaError_t launch_svd_rank(const double* R, const int64_t* d_rows, int64_t d, d
     int cg = (int)((d * d + 255) / 256);
     if (cg > 152 * 8) cg = 152 * 8;
     k_split_rows<<<cg, 256, 0, st>>>(R, d * d, Yh, Yl);
-    unsigned* barrier = work;
-    unsigned* rotated = work + 1;
-    if ((e = cudaMemsetAsync(work, 0, sizeof(unsigned) * (1 + kMaxSweeps), st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(version, 0, sizeof(unsigned) * (size_t)d, st)) != cudaSuccess) return e;
-    int di = (int)d, ms = kMaxSweeps;
-    void* kargs[] = {&Yh, &Yl, (void*)&d_rows, &di, &ms, &rotated, &barrier, &version, &status, &sweeps_out};
-    const void* fn = d <= 256 ? (const void*)k_jacobi_rows<1>
-                   : d <= 512 ? (const void*)k_jacobi_rows<2> : (const void*)k_jacobi_rows<4>;
-    int occ = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, 0)) != cudaSuccess) return e;
-    int grid = (int)((d + 1) / 2);                      // one CTA a pair where they fit
-    const int cap = num_sms * (occ < 1 ? 1 : occ);
-    if (grid > cap) grid = cap;
-    if (grid < 1) grid = 1;
-    if ((e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(256), kargs, 0, st)) != cudaSuccess) return e;
+    // one cluster of 1 to 16 CTAs (blocks of at least 8 rows) where its shared memory holds the rows twice
+    const int C = d <= 16 ? 1 : d <= 32 ? 2 : d <= 64 ? 4 : d <= 128 ? 8 : 16;
+    e = d <= 128 ? launch_jacobi_cluster<1>(Yh, Yl, d_rows, (int)d, C, kMaxSweeps, sweeps_out, st)
+      : d <= 256 ? launch_jacobi_cluster<2>(Yh, Yl, d_rows, (int)d, C, kMaxSweeps, sweeps_out, st)
+      : d <= 384 ? launch_jacobi_cluster<3>(Yh, Yl, d_rows, (int)d, C, kMaxSweeps, sweeps_out, st)
+                 : cudaErrorNotSupported;
+    if (e != cudaSuccess && e != cudaErrorNotSupported) return e;
+    if (e == cudaErrorNotSupported) {
+        unsigned* barrier = work;
+        unsigned* rotated = work + 1;
+        if ((e = cudaMemsetAsync(work, 0, sizeof(unsigned) * (1 + kMaxSweeps), st)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(version, 0, sizeof(unsigned) * (size_t)d, st)) != cudaSuccess) return e;
+        int di = (int)d, ms = kMaxSweeps;
+        void* kargs[] = {&Yh, &Yl, (void*)&d_rows, &di, &ms, &rotated, &barrier, &version, &status, &sweeps_out};
+        const void* fn = d <= 256 ? (const void*)k_jacobi_rows<1>
+                       : d <= 512 ? (const void*)k_jacobi_rows<2> : (const void*)k_jacobi_rows<4>;
+        int occ = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, 0)) != cudaSuccess) return e;
+        int grid = (int)((d + 1) / 2);                      // one CTA a pair where they fit
+        const int cap = num_sms * (occ < 1 ? 1 : occ);
+        if (grid > cap) grid = cap;
+        if (grid < 1) grid = 1;
+        if ((e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(256), kargs, 0, st)) != cudaSuccess) return e;
+    }
     k_join_rows<<<cg, 256, 0, st>>>(Yh, Yl, d * d, Y);
     k_sigma_rank<<<1, 1024, 0, st>>>(Y, d_rows, (int)d, tau, sigma, order, rank_out);
     return cudaGetLastError();
