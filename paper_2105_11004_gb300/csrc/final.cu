@@ -5,11 +5,13 @@
 // leaves registers: each CTA squares and sums its tile rows in the epilogue
 // (warp shuffles) and writes only theta~ (n floats).
 //
-// Dense: 64-row x 256-column register tile, 8 x 8 per thread, A and Mfull
-// staged through shared memory in 16-wide k slices (two stages).
+// Dense: 128-row (64 for small n) x 256-column register tile, 16 x 8 per
+// thread, A and Mfull staged through shared memory in 16-wide k slices (two
+// stages), packed FP32 FMAs on row pairs.
 // CSR: one warp per row (product form of Lemma 1): the warp broadcasts each
 // (col, val) of the row and every lane accumulates 8 columns of
 // val * Mfull[col, :] with 128-bit loads; then squares and warp-sums.
+#include "f32x2.cuh"
 #include "lev_common.cuh"
 #include "lev_kernels.cuh"
 
@@ -17,41 +19,50 @@ namespace lev {
 
 namespace {
 
-constexpr int FD_BM = 64, FD_BN = 256, FD_BK = 16;
+constexpr int FD_BN = 256, FD_BK = 16;
 
-template <bool VEC>
-__global__ void __launch_bounds__(256) k_final_dense_fp32(
+// A warp owns 2 NP rows (NP packed pairs), lane l columns 4 l .. + 3 and 128 + 4 l .. + 3. Bound by the FP32
+// FMA pipe: with 8 rows a thread (NP = 4) the columns' shared-memory reads, eight wavefronts for 64 FMAs a
+// lane, kept the pipe at 0.44 (2.88 ms at 1e6 x 256 x 256); 16 rows halve them. Row pairs are
+// packed because the rows' entries are read as pairs anyway (one broadcast a pair); the columns' entries are
+// doubled in registers. NP = 4 keeps small n on more SMs. Each sum runs over k in order, as scalar FMAs would.
+template <bool VEC, int NP>
+__global__ void __launch_bounds__(256, NP == 8 ? 1 : 2) k_final_dense_fp32(
         const float* __restrict__ A, int64_t lda, int64_t n, int d,
         const float* __restrict__ M, int k, float* __restrict__ theta) {
-    __shared__ __align__(16) float As[2][FD_BK][FD_BM];
+    constexpr int BM = 16 * NP, LD = BM + 4;               // rows of the tile; + 4: the transposed stores' banks
+    __shared__ __align__(16) float As[2][FD_BK][LD];
     __shared__ __align__(16) float Ms[2][FD_BK][FD_BN];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int64_t row0 = (int64_t)blockIdx.x * FD_BM;
-    // loader coordinates: A tile 64 x 16 (one float4 per thread), M tile 16 x 256 (4 float4)
+    const int64_t row0 = (int64_t)blockIdx.x * BM;
+    // loader coordinates: A tile BM x 16 (NP / 4 float4 per thread), M tile 16 x 256 (4 float4)
     const int a_r = t >> 2, a_c = (t & 3) * 4;
     const int m_r = t >> 4, m_c = (t & 15) * 4;
-    float th[8];
+    float th[2 * NP];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) th[i] = 0.f;
+    for (int i = 0; i < 2 * NP; ++i) th[i] = 0.f;
 
     for (int q0 = 0; q0 < k; q0 += FD_BN) {
-        float acc[8][8];
+        f32x2 acc[NP][8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < NP; ++i)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-        float ra[4], rm[4][4];
+            for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
+        float ra[NP / 4][4], rm[4][4];
         auto load = [&](int k0) {
-            const int64_t gr = row0 + a_r;
-            if (VEC) {
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (gr < n && k0 + a_c < d) v = __ldg(reinterpret_cast<const float4*>(A + gr * lda + k0 + a_c));
-                ra[0] = v.x; ra[1] = v.y; ra[2] = v.z; ra[3] = v.w;
-            } else {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int c = k0 + a_c + i;
-                    ra[i] = (gr < n && c < d) ? __ldg(A + gr * lda + c) : 0.f;
+            for (int u = 0; u < NP / 4; ++u) {
+                const int64_t gr = row0 + a_r + 64 * u;
+                if (VEC) {
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (gr < n && k0 + a_c < d) v = __ldg(reinterpret_cast<const float4*>(A + gr * lda + k0 + a_c));
+                    ra[u][0] = v.x; ra[u][1] = v.y; ra[u][2] = v.z; ra[u][3] = v.w;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int c = k0 + a_c + i;
+                        ra[u][i] = (gr < n && c < d) ? __ldg(A + gr * lda + c) : 0.f;
+                    }
                 }
             }
             const int mr = k0 + m_r;
@@ -71,7 +82,9 @@ __global__ void __launch_bounds__(256) k_final_dense_fp32(
         };
         auto store = [&](int st) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) As[st][a_c + i][a_r] = ra[i];
+            for (int u = 0; u < NP / 4; ++u)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) As[st][a_c + i][a_r + 64 * u] = ra[u][i];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 *reinterpret_cast<float4*>(&Ms[st][m_r][m_c + 64 * u]) =
@@ -87,16 +100,22 @@ __global__ void __launch_bounds__(256) k_final_dense_fp32(
             if (more) load(k0 + FD_BK);
 #pragma unroll
             for (int kk = 0; kk < FD_BK; ++kk) {
-                const float4 a0 = *reinterpret_cast<const float4*>(&As[st][kk][w * 4]);
-                const float4 a1 = *reinterpret_cast<const float4*>(&As[st][kk][32 + w * 4]);
+                f32x2 a[NP];
+#pragma unroll
+                for (int i = 0; i < NP; i += 2) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&As[st][kk][w * 2 * NP + 2 * i]);
+                    a[i] = v.x;
+                    a[i + 1] = v.y;
+                }
                 const float4 b0 = *reinterpret_cast<const float4*>(&Ms[st][kk][lane * 4]);
                 const float4 b1 = *reinterpret_cast<const float4*>(&Ms[st][kk][128 + lane * 4]);
-                const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
                 const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                for (int j = 0; j < 8; ++j) {
+                    const f32x2 bb = pack2(b[j], b[j]);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                    for (int i = 0; i < NP; ++i) acc[i][j] = fma2(a[i], bb, acc[i][j]);
+                }
             }
             if (more) {
                 store(st ^ 1);
@@ -105,17 +124,20 @@ __global__ void __launch_bounds__(256) k_final_dense_fp32(
             }
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float sq = 0.f;
+        for (int i = 0; i < NP; ++i) {
+            f32x2 sq = 0ull;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) sq = fmaf(acc[i][j], acc[i][j], sq);
-            th[i] += sq;
+            for (int j = 0; j < 8; ++j) sq = fma2(acc[i][j], acc[i][j], sq);
+            float s0, s1;
+            unpack2(sq, s0, s1);
+            th[2 * i] += s0;
+            th[2 * i + 1] += s1;
         }
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < 2 * NP; ++i) {
         const float v = warp_sum(th[i]);
-        const int64_t r = row0 + (i < 4 ? w * 4 + i : 32 + w * 4 + (i - 4));
+        const int64_t r = row0 + w * 2 * NP + i;
         if (lane == 0 && r < n) theta[r] = v;
     }
 }
@@ -369,12 +391,19 @@ cudaError_t launch_final_dense_fp32(const float* A, int64_t lda, int64_t n, int6
                                     const float* Mfull, int64_t k, float* theta, cudaStream_t st) {
     const bool vec = (reinterpret_cast<uintptr_t>(A) % 16 == 0) && (reinterpret_cast<uintptr_t>(Mfull) % 16 == 0) &&
                      (lda % 4 == 0) && (d % 4 == 0) && (k % 4 == 0);
-    const int64_t grid = (n + FD_BM - 1) / FD_BM;
+    // 128 rows a CTA, one CTA an SM; below two rounds of them, 64 rows and two CTAs an SM
+    const bool big = n >= 2 * 152 * 128;
+    const int64_t bm = big ? 128 : 64, grid = (n + bm - 1) / bm;
     if (grid > 0x7fffffff) return cudaErrorInvalidValue;
-    if (vec)
-        k_final_dense_fp32<true><<<(unsigned)grid, 256, 0, st>>>(A, lda, n, (int)d, Mfull, (int)k, theta);
+    const unsigned g = (unsigned)grid;
+    if (vec && big)
+        k_final_dense_fp32<true, 8><<<g, 256, 0, st>>>(A, lda, n, (int)d, Mfull, (int)k, theta);
+    else if (vec)
+        k_final_dense_fp32<true, 4><<<g, 256, 0, st>>>(A, lda, n, (int)d, Mfull, (int)k, theta);
+    else if (big)
+        k_final_dense_fp32<false, 8><<<g, 256, 0, st>>>(A, lda, n, (int)d, Mfull, (int)k, theta);
     else
-        k_final_dense_fp32<false><<<(unsigned)grid, 256, 0, st>>>(A, lda, n, (int)d, Mfull, (int)k, theta);
+        k_final_dense_fp32<false, 4><<<g, 256, 0, st>>>(A, lda, n, (int)d, Mfull, (int)k, theta);
     return cudaGetLastError();
 }
 

@@ -11,6 +11,9 @@
 //    reduction of the split partials (tensor-core forms live in tc_sketch.cu).
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
+#include "f32x2.cuh"
 #include "lev_common.cuh"
 #include "lev_kernels.cuh"
 
@@ -482,6 +485,106 @@ __global__ void __launch_bounds__(256) k_sgemm_splitk(
     }
 }
 
+// The same product with a 128 x 256 tile, 16 x 8 outputs per thread as packed row pairs (the loop of
+// k_final_dense_fp32: half the shared-memory reads a product of the 8 x 8 tile, which kept the FMA pipe at
+// 0.44), 16-byte loads: N > 128, K and N multiples of 4, 16-byte aligned operands. kchunk is a multiple of 16.
+constexpr int SW_BM = 128, SW_BN = 256, SW_BK = 16;
+
+__global__ void __launch_bounds__(256, 1) k_sgemm_splitk_wide(
+        const float* __restrict__ G, const float* __restrict__ B, int M, int N, int64_t K,
+        int64_t kchunk, float* __restrict__ P) {
+    __shared__ __align__(16) float As[2][SW_BK][SW_BM + 4];
+    __shared__ __align__(16) float Bs[2][SW_BK][SW_BN];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int m0 = blockIdx.y * SW_BM, n0 = blockIdx.x * SW_BN;
+    const int64_t kb = (int64_t)blockIdx.z * kchunk, ke = min(K, kb + kchunk);
+    const int a_r = t >> 2, a_c = (t & 3) * 4;             // two float4 of G: rows a_r and a_r + 64
+    const int b_r = t >> 4, b_c = (t & 15) * 4;            // four float4 of B
+    f32x2 acc[8][8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
+    float4 ra[2], rb[4];
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto load = [&](int64_t k0) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int r = m0 + a_r + 64 * u;
+            ra[u] = (r < M && k0 + a_c < ke) ? __ldg(reinterpret_cast<const float4*>(G + (int64_t)r * K + k0 + a_c)) : zero;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c = n0 + b_c + 64 * u;
+            rb[u] = (k0 + b_r < ke && c < N) ? __ldg(reinterpret_cast<const float4*>(B + (k0 + b_r) * N + c)) : zero;
+        }
+    };
+    auto store = [&](int st) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            As[st][a_c][a_r + 64 * u] = ra[u].x;
+            As[st][a_c + 1][a_r + 64 * u] = ra[u].y;
+            As[st][a_c + 2][a_r + 64 * u] = ra[u].z;
+            As[st][a_c + 3][a_r + 64 * u] = ra[u].w;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) *reinterpret_cast<float4*>(&Bs[st][b_r][b_c + 64 * u]) = rb[u];
+    };
+    int st = 0;
+    if (kb < ke) {
+        load(kb);
+        store(0);
+    }
+    __syncthreads();
+    for (int64_t k0 = kb; k0 < ke; k0 += SW_BK) {
+        const bool more = k0 + SW_BK < ke;
+        if (more) load(k0 + SW_BK);
+#pragma unroll
+        for (int kk = 0; kk < SW_BK; ++kk) {
+            f32x2 a[8];
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&As[st][kk][w * 16 + 2 * i]);
+                a[i] = v.x;
+                a[i + 1] = v.y;
+            }
+            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[st][kk][lane * 4]);
+            const float4 b1 = *reinterpret_cast<const float4*>(&Bs[st][kk][128 + lane * 4]);
+            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const f32x2 bb = pack2(b[j], b[j]);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[i][j] = fma2(a[i], bb, acc[i][j]);
+            }
+        }
+        if (more) {
+            store(st ^ 1);
+            __syncthreads();
+            st ^= 1;
+        }
+    }
+    float* out = P + (int64_t)blockIdx.z * M * N;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        float y[2][8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) unpack2(acc[i][j], y[0][j], y[1][j]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int row = m0 + w * 16 + 2 * i + u;
+            if (row >= M) continue;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int c = n0 + 128 * q + lane * 4;
+                if (c < N)
+                    *reinterpret_cast<float4*>(out + (int64_t)row * N + c) =
+                        make_float4(y[u][4 * q], y[u][4 * q + 1], y[u][4 * q + 2], y[u][4 * q + 3]);
+            }
+        }
+    }
+}
+
 __global__ void k_reduce_splits(const float* __restrict__ P, int splits, int64_t count,
                                 float* __restrict__ out) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -611,10 +714,18 @@ cudaError_t launch_gen_gaussian(int64_t m, int64_t s, int64_t ld, uint64_t seed,
     return cudaGetLastError();
 }
 
+static bool sgemm_wide(int64_t d, int64_t s) { return d > 128 && d % 4 == 0 && s % 4 == 0; }
+
+// Split-K of the FP32 stage: two waves of the wide tile (one CTA an SM) or about four 128 x 128 tiles an SM, which
+// is the same length of an FP32 chain; at least 256 k a split, 64 where that leaves SMs idle (m = 80, d = 20,
+// s = 1,600: 30 us on 7 CTAs).
 int gaussian_stage_splits(int64_t m, int64_t d, int64_t s) {
-    const int64_t tiles = ((m + SG_BM - 1) / SG_BM) * ((d + SG_BN - 1) / SG_BN);
-    int64_t splits = (152 * 4 + tiles - 1) / tiles;          // about 4 CTAs per SM
-    const int64_t max_by_k = (s + 255) / 256;                 // at least 256 k per split
+    const bool wide = sgemm_wide(d, s);
+    const int64_t tiles = wide ? ((m + SW_BM - 1) / SW_BM) * ((d + SW_BN - 1) / SW_BN)
+                               : ((m + SG_BM - 1) / SG_BM) * ((d + SG_BN - 1) / SG_BN);
+    int64_t splits = wide ? std::max<int64_t>(1, 304 / tiles) : (608 + tiles - 1) / tiles;
+    const int64_t per = ((s + 255) / 256) * tiles >= 152 ? 256 : 64;
+    const int64_t max_by_k = (s + per - 1) / per;
     if (splits > max_by_k) splits = max_by_k;
     if (splits < 1) splits = 1;
     return (int)splits;
@@ -624,9 +735,16 @@ cudaError_t launch_gaussian_stage_fp32(const float* G, const float* B, int64_t m
                                        int64_t d, float* partial, int splits, float* Atilde,
                                        cudaStream_t st) {
     int64_t kchunk = (s + splits - 1) / splits;
-    kchunk = (kchunk + SG_BK - 1) / SG_BK * SG_BK;
-    dim3 grid((unsigned)((d + SG_BN - 1) / SG_BN), (unsigned)((m + SG_BM - 1) / SG_BM), (unsigned)splits);
-    k_sgemm_splitk<<<grid, 256, 0, st>>>(G, B, (int)m, (int)d, s, kchunk, partial);
+    // G, B and the partials are buffers of the handle (256-byte aligned)
+    if (sgemm_wide(d, s)) {
+        kchunk = (kchunk + SW_BK - 1) / SW_BK * SW_BK;
+        dim3 grid((unsigned)((d + SW_BN - 1) / SW_BN), (unsigned)((m + SW_BM - 1) / SW_BM), (unsigned)splits);
+        k_sgemm_splitk_wide<<<grid, 256, 0, st>>>(G, B, (int)m, (int)d, s, kchunk, partial);
+    } else {
+        kchunk = (kchunk + SG_BK - 1) / SG_BK * SG_BK;
+        dim3 grid((unsigned)((d + SG_BN - 1) / SG_BN), (unsigned)((m + SG_BM - 1) / SG_BM), (unsigned)splits);
+        k_sgemm_splitk<<<grid, 256, 0, st>>>(G, B, (int)m, (int)d, s, kchunk, partial);
+    }
     k_reduce_splits<<<grid_for(m * d, 256, 152 * 8), 256, 0, st>>>(partial, splits, m * d, Atilde);
     return cudaGetLastError();
 }
