@@ -23,6 +23,7 @@
 
 #include <algorithm>
 
+#include "f32x2.cuh"
 #include "lev_common.cuh"
 #include "lev_kernels.cuh"
 
@@ -61,11 +62,11 @@ __global__ void __launch_bounds__(256) k_bwd_wgram(const float* __restrict__ A, 
     const int t = threadIdx.x, g = t >> 6, tt = t & 63, ti = tt >> 3, tj = tt & 7;
     const int64_t r_begin = (int64_t)blockIdx.x * rows_per_chunk;
     const int64_t r_end = min(n, r_begin + rows_per_chunk);
-    float acc[8][8];
+    f32x2 acc[8][4];                        // columns 2 v, 2 v + 1 of the thread's eight
 #pragma unroll
     for (int u = 0; u < 8; ++u)
 #pragma unroll
-        for (int v = 0; v < 8; ++v) acc[u][v] = 0.f;
+        for (int v = 0; v < 4; ++v) acc[u][v] = 0ull;
     for (int64_t r0 = r_begin; r0 < r_end; r0 += H_RB) {
         __syncthreads();
         // 32 rows x 64 columns per side; float4 loads when A is 16-byte aligned and lda % 4 == 0
@@ -97,14 +98,16 @@ __global__ void __launch_bounds__(256) k_bwd_wgram(const float* __restrict__ A, 
             const float wr = ws[r];
             const float4 a0 = *reinterpret_cast<const float4*>(Ai + r * HT + ti * 8);
             const float4 a1 = *reinterpret_cast<const float4*>(Ai + r * HT + ti * 8 + 4);
-            const float4 b0 = *reinterpret_cast<const float4*>(Aj + r * HT + tj * 8);
-            const float4 b1 = *reinterpret_cast<const float4*>(Aj + r * HT + tj * 8 + 4);
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(Aj + r * HT + tj * 8);
+            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(Aj + r * HT + tj * 8 + 4);
             const float av[8] = {wr * a0.x, wr * a0.y, wr * a0.z, wr * a0.w, wr * a1.x, wr * a1.y, wr * a1.z, wr * a1.w};
-            const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+            const f32x2 bv[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
+            for (int u = 0; u < 8; ++u) {
+                const f32x2 a2 = pack2(av[u], av[u]);
 #pragma unroll
-                for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
+                for (int v = 0; v < 4; ++v) acc[u][v] = fma2(a2, bv[v], acc[u][v]);
+            }
         }
     }
     // the four groups' blocks, summed in a fixed order
@@ -113,7 +116,8 @@ __global__ void __launch_bounds__(256) k_bwd_wgram(const float* __restrict__ A, 
 #pragma unroll
     for (int u = 0; u < 8; ++u)
 #pragma unroll
-        for (int v = 0; v < 8; ++v) red[(g * HT + ti * 8 + u) * HT + tj * 8 + v] = acc[u][v];
+        for (int v = 0; v < 4; ++v)
+            *reinterpret_cast<f32x2*>(red + (g * HT + ti * 8 + u) * HT + tj * 8 + 2 * v) = acc[u][v];
     __syncthreads();
     float* out = Hp + ((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * (HT * HT);
     for (int e = t; e < HT * HT; e += 256)
@@ -338,11 +342,11 @@ __global__ void __launch_bounds__(256) k_bwd_pass2(const float* __restrict__ A, 
     const int t = threadIdx.x, tr = t >> 4, tc = t & 15;
     const int64_t r0 = (int64_t)blockIdx.x * P2_R;
     const int c0 = blockIdx.y * P2_C;
-    float acc[8][4];
+    f32x2 acc[8][2];                         // columns 2 v, 2 v + 1 of the thread's four
 #pragma unroll
     for (int u = 0; u < 8; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
+        for (int v = 0; v < 2; ++v) acc[u][v] = 0ull;
     for (int j0 = 0; j0 < d; j0 += P2_J) {
         __syncthreads();
         for (int e = t; e < P2_R * (P2_J / 4); e += 256) {
@@ -377,20 +381,20 @@ __global__ void __launch_bounds__(256) k_bwd_pass2(const float* __restrict__ A, 
         __syncthreads();
 #pragma unroll 2
         for (int j = 0; j < P2_J; j += 4) {
-            float4 a[8], p[4];
+            float4 a[8];
+            ulonglong2 p[4];
 #pragma unroll
             for (int u = 0; u < 8; ++u) a[u] = *reinterpret_cast<const float4*>(As + (tr * 8 + u) * P2_AS + j);
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) p[jj] = *reinterpret_cast<const float4*>(Ps + (j + jj) * P2_C + tc * 4);
+            for (int jj = 0; jj < 4; ++jj) p[jj] = *reinterpret_cast<const ulonglong2*>(Ps + (j + jj) * P2_C + tc * 4);
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const float av[4] = {a[u].x, a[u].y, a[u].z, a[u].w};
 #pragma unroll
                 for (int jj = 0; jj < 4; ++jj) {
-                    acc[u][0] = fmaf(av[jj], p[jj].x, acc[u][0]);
-                    acc[u][1] = fmaf(av[jj], p[jj].y, acc[u][1]);
-                    acc[u][2] = fmaf(av[jj], p[jj].z, acc[u][2]);
-                    acc[u][3] = fmaf(av[jj], p[jj].w, acc[u][3]);
+                    const f32x2 a2 = pack2(av[jj], av[jj]);
+                    acc[u][0] = fma2(a2, p[jj].x, acc[u][0]);
+                    acc[u][1] = fma2(a2, p[jj].y, acc[u][1]);
                 }
             }
         }
@@ -406,9 +410,12 @@ __global__ void __launch_bounds__(256) k_bwd_pass2(const float* __restrict__ A, 
         const float tw = 2.f * w[row];
         const float* trow = T + bucket * d;
         float* out = gA + row * d;
+        float y[4];
+        unpack2(acc[u][0], y[0], y[1]);
+        unpack2(acc[u][1], y[2], y[3]);
 #pragma unroll
         for (int v = 0; v < 4; ++v)
-            if (c + v < d) out[c + v] = fmaf(tw, acc[u][v], sg * trow[c + v]);
+            if (c + v < d) out[c + v] = fmaf(tw, y[v], sg * trow[c + v]);
     }
 }
 

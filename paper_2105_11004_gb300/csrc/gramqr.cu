@@ -43,6 +43,7 @@
 #include <climits>
 
 #include "df.cuh"
+#include "f32x2.cuh"
 #include "lev_common.cuh"
 #include "lev_kernels.cuh"
 
@@ -90,25 +91,32 @@ __global__ void __launch_bounds__(256) k_gram_dot2(const float* __restrict__ At,
             Bs[r][c] = (rok && bj * GT + c < d) ? At[(int64_t)row * lda + bj * GT + c] : 0.f;
         }
         __syncthreads();
-        float sm[4] = {0.f, 0.f, 0.f, 0.f}, cm[4] = {0.f, 0.f, 0.f, 0.f};
+        f32x2 sm[2] = {0ull, 0ull}, cm[2] = {0ull, 0ull};    // two outputs an instruction
 #pragma unroll 8
         for (int r = 0; r < kDot2Rows; ++r) {
-            const float a = As[r][ty];
-            const float4 b4 = *reinterpret_cast<const float4*>(&Bs[r][tx * 4]);
-            const float bq[4] = {b4.x, b4.y, b4.z, b4.w};
+            const float a1 = As[r][ty];
+            const f32x2 a = pack2(a1, a1);
+            const ulonglong2 b4 = *reinterpret_cast<const ulonglong2*>(&Bs[r][tx * 4]);
+            const f32x2 bq[2] = {b4.x, b4.y};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float p = __fmul_rn(a, bq[q]);
-                const float ep = __fmaf_rn(a, bq[q], -p);          // a b = p + ep exactly
-                const float s1 = __fadd_rn(sm[q], p);
-                const float z = __fsub_rn(s1, sm[q]);
-                const float es = __fadd_rn(__fsub_rn(sm[q], __fsub_rn(s1, z)), __fsub_rn(p, z));  // s + p = s1 + es
+            for (int q = 0; q < 2; ++q) {
+                const f32x2 p = mul2(a, bq[q]);
+                const f32x2 ep = fma2(a, bq[q], neg2(p));          // a b = p + ep exactly
+                const f32x2 s1 = add2(sm[q], p);
+                const f32x2 z = sub2(s1, sm[q]);
+                const f32x2 es = add2(sub2(sm[q], sub2(s1, z)), sub2(p, z));  // s + p = s1 + es
                 sm[q] = s1;
-                cm[q] = __fadd_rn(cm[q], __fadd_rn(es, ep));
+                cm[q] = add2(cm[q], add2(es, ep));
             }
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] += (double)sm[q] + (double)cm[q];
+        for (int q = 0; q < 2; ++q) {
+            float s0, s1, c0, c1;
+            unpack2(sm[q], s0, s1);
+            unpack2(cm[q], c0, c1);
+            acc[2 * q] += (double)s0 + (double)c0;
+            acc[2 * q + 1] += (double)s1 + (double)c1;
+        }
         __syncthreads();
     }
     double* out = Gp + ((int64_t)split * T + blockIdx.x) * (GT * GT);
