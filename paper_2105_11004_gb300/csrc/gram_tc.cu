@@ -10,32 +10,36 @@
 //     (i > 0: at most half a unit of digit i - 1). Each t_i is a BF16 number; what is left after the seventh
 //     digit is below 2^-56 of the column's largest entry (a 24-bit entry leaves nothing unless it is
 //     smaller than 2^-32 of it);
-//   * the products t_i t_j with i + j = g are multiples of 2^(-8g) of at most 2^(14 - 8g), g + 1 pairs of
-//     them a row: over a chunk of 192 rows the sum stays inside 24 bits for g <= 4 ((g + 1) 192 <= 1024), so
-//     the accumulators of g = 0 .. 4 are exact; those of g = 5 and 6 share one accumulator, whose FP32
-//     rounding (below 2^-24 of a sum of weight 2^-40) is beyond the digits kept. Pairs with i + j > 6 are
-//     dropped (2^-56);
-//   * every 192 rows the accumulators join a running FP32 pair per entry of the tile, and the partial sums of
+//   * the products t_i t_j with i + j = g are multiples of 2^(-8g) of at most 2^(14 - 8g). A 24-bit entry has
+//     at most four digits that are not zero, in a row (its first at i0: it is at least 2^(-8 i0 - 1), a multiple
+//     of 2^(-8 i0 - 24), so digit i0 + 3 leaves nothing), so a row has at most four of these products, and over
+//     a chunk of 256 rows the sum stays inside 24 bits: the accumulators of g = 0 .. 6 are exact. Pairs with
+//     i + j > 6 are dropped (2^-56);
+//   * every 256 rows the accumulators join a running FP32 pair per entry of the tile, and the partial sums of
 //     the row splits are scaled back (powers of two) and added in FP64 in a fixed order.
 // Measured against a 64-bit product, relative to sqrt(G_ii G_jj) and through the factor R^T R (whose own
 // rounding is about 5e-14): 7.2e-14 at 4096 x 1024 Gaussian (7.5e-14 with the compensated sums), 1.8e-14 with
 // rows scaled by e^(2 N) (8.4e-14), 1.7e-14 at 4096 x 500 with e^(4 N) (4.7e-14), 2.3e-14 with one row 1e4
 // times the others (1.6e-13).
 //
-// One CTA takes a 128 x 128 tile of G over a range of rows. A tile of the diagonal needs only the pairs
-// i <= j: X = sum_{i<j} T_i^T T_j + sum_i T_i^T (T_i / 2) and G = X + X^T (16 MMAs a K step of 16 rows
-// instead of 28), so it gets fewer splits. 512 accumulator columns hold four 128 x 128 accumulators, and
-// six are needed: a chunk runs twice through the ring of stages, first for g = 0 .. 3 (four digits),
-// then for g = 4 and g = 5, 6 (seven digits); converting twice costs less than smaller tiles, whose MMAs
-// would wait for shared memory (a 128 x 128 x 16 MMA already reads its 128 bytes a cycle).
+// Equal columns give bitwise equal rows and columns of G, as the symmetric compensated sums do (a pivot tie
+// goes to the lower index): the chunk sums are exact, and every tile has the same chunks and row splits, so
+// an entry's roundings do not depend on the tile it lies in.
+//
+// One CTA takes a 128 x 128 tile of G over a range of rows. 512 accumulator columns hold four 128 x 128
+// accumulators, and seven are needed: a chunk runs twice through the ring of stages, first for g = 0 .. 3 (four
+// digits), then for g = 4 .. 6 (seven digits); converting twice costs less than smaller tiles, whose MMAs
+// would wait for shared memory (a 128 x 128 x 16 MMA already reads its 128 bytes a cycle). A tile of the
+// diagonal has one operand to convert and takes three quarters of the time of another.
 //   * warps 8..15 (converters): thread = column; read 16 rows of the column two half steps ahead (cp.async,
 //     any alignment), cut them into digits and store each digit's 16-byte pieces into the stage (K-major rows
 //     of 32 bytes, 32-byte swizzle);
 //   * warp 16: allocates tensor memory and issues the MMAs (M = N = 128, K = 16);
 //   * warps 0..7 (fetchers): TMEM lane = row of the tile, 64 columns a warp; add a pass's accumulators to the
 //     running pairs and hand each accumulator back as soon as it is read.
-// The converters' issue slots set the pace (tensor pipe 40% active): 2.07 ms at 1e6 x 256, with the column
-// maxima 0.17 ms and the sum of the splits 0.02 ms, against 17.1 ms for the compensated sums; 0.15 + 0.03 ms
+// The converters set the pace (two warps a scheduler; the MMAs are 48% of a tile's time above the diagonal):
+// 2.05 ms at 1e6 x 256, with the column maxima 0.17 ms and the sum of the splits 0.03 ms, against 17.1 ms for
+// the compensated sums; 0.15 + 0.03 ms
 // at 4096 x 1024 against 1.03 ms. Every wait is bounded; after a timeout the CTA runs on without waiting (its
 // barriers stay matched) and records the failure in the status word.
 #include <atomic>
@@ -62,7 +66,7 @@ constexpr int kFetchWarps = 8, kConvWarps = 8;               // two warpgroups e
 constexpr int kMmaWarp = kFetchWarps + kConvWarps;
 constexpr int kThreads = (kMmaWarp + 4) * 32;
 constexpr int kConvThreads = kConvWarps * 32;
-constexpr int kMaxChunk = 192;
+constexpr int kMaxChunk = 256;
 constexpr int kHalf = 8;                                    // rows of its column a worker converts at a time
 constexpr int kRing = 3;                                   // half steps of a thread's column, read two ahead
 constexpr int kSlotFloats = kHalf * kConvThreads;
@@ -129,10 +133,9 @@ __device__ __forceinline__ void store_digit(uint8_t* dst, const f32x2 (&t)[4]) {
     *reinterpret_cast<uint4*>(dst) = v;
 }
 
-// Eight scaled entries into N digits (slice q at dst + q * slice_bytes); `half`: also digits H0 and H0 + 1
-// halved, as slices 7 + H0 and 8 + H0 (a diagonal tile's second operand).
-template <int N, int H0>
-__device__ __forceinline__ void cut_digits(f32x2 (&y)[4], uint8_t* dst, int slice_bytes, bool half) {
+// Eight scaled entries into N digits (slice q at dst + q * slice_bytes).
+template <int N>
+__device__ __forceinline__ void cut_digits(f32x2 (&y)[4], uint8_t* dst, int slice_bytes) {
     float magic = 12582912.0f;                             // 1.5 2^23: y + magic - magic rounds y to an integer
 #pragma unroll
     for (int q = 0; q < N; ++q) {
@@ -144,21 +147,14 @@ __device__ __forceinline__ void cut_digits(f32x2 (&y)[4], uint8_t* dst, int slic
             if (q + 1 < N) y[k] = sub2(y[k], t[k]);
         }
         store_digit(dst + q * slice_bytes, t);
-        if (half && (q == H0 || q == H0 + 1)) {
-            const f32x2 hf = pack2(0.5f, 0.5f);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) t[k] = mul2(t[k], hf);
-            store_digit(dst + (7 + q) * slice_bytes, t);
-        }
         magic *= 0.00390625f;
     }
 }
 
 struct GramPlan {
     int nt, noff;              // 128-column blocks, tiles above the diagonal
-    int so, sd;                // row splits of a tile above / on the diagonal
-    int rows_o, rows_d;        // rows a split
-    int chunk_o, chunk_d;      // rows a chunk (multiple of 16, at most 192)
+    int splits, rows;          // row splits of every tile, rows a split
+    int chunk;                 // rows a chunk (multiple of 16, at most kMaxChunk)
 };
 
 __device__ __forceinline__ void off_tile(int t, int nt, int& bi, int& bj) {
@@ -167,8 +163,7 @@ __device__ __forceinline__ void off_tile(int t, int nt, int& bi, int& bj) {
     bj = bi + 1 + t;
 }
 
-// The MMAs of one K step for pass 0 (g = 0 .. 3, accumulator g) or pass 1 (g = 4 into accumulator 0, g = 6
-// and 5 into accumulator 1). sa: stage address (digit 0 of the tile's rows); the operands of the tile's
+// The MMAs of one K step for pass 0 (g = 0 .. 3, accumulator g) or pass 1 (g = 4 .. 6, accumulator g - 4). sa: stage address (digit 0 of the tile's rows); the operands of the tile's
 // columns follow them, or are the same rows (a tile of the diagonal). `first`: the pass's first step (the
 // accumulators start at zero, and each is waited for). One thread issues them, so the operand
 // addresses are constants off one descriptor.
@@ -192,18 +187,14 @@ template <bool DIAG, int PASS, class WaitAcc>
 __device__ __forceinline__ void issue_step(uint32_t lead, uint32_t sa, uint32_t tmem, bool first, WaitAcc wait_acc) {
     constexpr uint32_t kSlice = (DIAG ? 1u : 2u) * kTile * 32u, idesc = make_idesc(false, kTile, kTile);
     const uint64_t a = sw32_desc(sa), b = a + (DIAG ? 0u : kTile * 32u / 16u);
-    constexpr int kGroups = PASS == 0 ? 4 : 3;
 #pragma unroll
-    for (int q = 0; q < kGroups; ++q) {
-        const int g = PASS == 0 ? q : (q == 0 ? 4 : 7 - q), acc = PASS == 0 ? q : (q == 0 ? 0 : 1);
-        const bool opens = PASS == 0 || q < 2;              // first group into its accumulator
-        if (opens && first) wait_acc(acc);
+    for (int acc = 0; acc < (PASS == 0 ? 4 : 3); ++acc) {
+        const int g = 4 * PASS + acc;
+        if (first) wait_acc(acc);
 #pragma unroll
-        for (int i = 0; i <= (DIAG ? g / 2 : g); ++i) {
-            const int j = g - i, bo = DIAG && i == j ? 7 + i : j;
-            mma_if(lead, tmem + (uint32_t)acc * kTile, a + (uint32_t)i * (kSlice / 16u), b + (uint32_t)bo * (kSlice / 16u),
-                          idesc, (opens && i == 0 && first) ? 0u : 1u);
-        }
+        for (int i = 0; i <= g; ++i)
+            mma_if(lead, tmem + (uint32_t)acc * kTile, a + (uint32_t)i * (kSlice / 16u), b + (uint32_t)(g - i) * (kSlice / 16u),
+                   idesc, (i == 0 && first) ? 0u : 1u);
     }
 }
 
@@ -244,21 +235,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(const float* __restrict
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     // unit: a tile and a range of rows; tiles above the diagonal first
-    int bi, bj, split, rows, K;
-    const bool diag = (int)blockIdx.x >= pl.noff * pl.so;
+    int bi, bj, split;
+    const bool diag = (int)blockIdx.x >= pl.noff * pl.splits;
     if (!diag) {
         split = (int)blockIdx.x / pl.noff;
         off_tile((int)blockIdx.x % pl.noff, pl.nt, bi, bj);
-        rows = pl.rows_o;
-        K = pl.chunk_o;
     } else {
-        const int u = (int)blockIdx.x - pl.noff * pl.so;
+        const int u = (int)blockIdx.x - pl.noff * pl.splits;
         split = u / pl.nt;
         bi = bj = u % pl.nt;
-        rows = pl.rows_d;
-        K = pl.chunk_d;
     }
-    const int64_t r_begin = min(m, (int64_t)split * rows), r_end = min(m, r_begin + rows);
+    const int K = pl.chunk;
+    const int64_t r_begin = min(m, (int64_t)split * pl.rows), r_end = min(m, r_begin + pl.rows);
     const int ns = K / 16;                                 // K steps a pass
     const int nchunk = (int)((r_end - r_begin + K - 1) / K);
     const int nseg = 2 * nchunk;                           // passes
@@ -417,8 +405,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(const float* __restrict
                         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(a1) : "r"(from + (2 * k + 1) * (kConvThreads * 4)) : "memory");
                         x[k] = mul2(pack2(a0, a1), sc);
                     }
-                    if (at.pass == 0) cut_digits<4, 0>(x, to + ((hh << 4) ^ swz), slice, diag);
-                    else cut_digits<kDigits, 2>(x, to + ((hh << 4) ^ swz), slice, diag);
+                    if (at.pass == 0) cut_digits<4>(x, to + ((hh << 4) ^ swz), slice);
+                    else cut_digits<kDigits>(x, to + ((hh << 4) ^ swz), slice);
                 }
                 if (++slot == kRing) slot = 0;
             }
@@ -446,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(const float* __restrict
             wait_or_abort(smem_u32(&ctl->tfull), (uint32_t)(seg & 1), ctl, status);
             __syncwarp();
             tc_fence_after();
-            const int nacc = pass == 0 ? 4 : 2;
+            const int nacc = pass == 0 ? 4 : 3;
             for (int a = 0; a < nacc; ++a) {
 #pragma unroll
                 for (int j0 = 0; j0 < 64; j0 += 8) {
@@ -458,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(const float* __restrict
                         __syncwarp();
                         if (lane == 0) {
                             mbar_arrive(smem_u32(&ctl->afree[a]));
-                            if (pass == 1) mbar_arrive(smem_u32(&ctl->afree[a + 2]));
+                            if (pass == 1 && a == 2) mbar_arrive(smem_u32(&ctl->afree[3]));
                         }
                     }
                     if (pass == 0) {
@@ -517,9 +505,9 @@ __device__ __forceinline__ double scaled_double(float x, int k) {
     return e == 0 ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
 }
 
-// G (d x d, both triangles) from the units' partials: scaled back and added in FP64, X + X^T for a tile of
-// the diagonal. A CTA takes a 32 x 4 block of a tile (blockIdx.y: block row + 4 block column); warp w adds
-// the splits w, w + 8, ... of its four columns, then the warps' sums are added in warp order.
+// G (d x d, both triangles) from the units' partials: scaled back and added in FP64. A CTA takes a 32 x 4
+// block of a tile (blockIdx.y: block row + 4 block column); warp w adds the splits w, w + 8, ... of its four
+// columns, then the warps' sums are added in warp order.
 __global__ void __launch_bounds__(256) k_gram_tc_reduce(const double* __restrict__ Gp, int d, GramPlan pl,
                                                         double* __restrict__ G) {
     constexpr int T = kTile * kTile;
@@ -530,13 +518,12 @@ __global__ void __launch_bounds__(256) k_gram_tc_reduce(const double* __restrict
     int bi, bj;
     if (diag) bi = bj = tile - pl.noff;
     else off_tile(tile, pl.nt, bi, bj);
-    const double* p = Gp + (int64_t)(diag ? pl.noff * pl.so + bi : tile) * kUnitDoubles;
+    const double* p = Gp + (int64_t)(diag ? pl.noff * pl.splits + bi : tile) * kUnitDoubles;
     const int64_t stride = (int64_t)(diag ? pl.nt : pl.noff) * kUnitDoubles;
-    const int splits = diag ? pl.sd : pl.so;
     const int tx = threadIdx.x & 31, w = threadIdx.x >> 5;
     double s[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 2
-    for (int z = w; z < splits; z += 8) {
+    for (int z = w; z < pl.splits; z += 8) {
         const double* u = p + z * stride;
         const int32_t* ex = reinterpret_cast<const int32_t*>(u + T);
         const int er = ex[r0 + tx] - 14;
@@ -544,25 +531,11 @@ __global__ void __launch_bounds__(256) k_gram_tc_reduce(const double* __restrict
         float2 x[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) x[q] = v[(c0 + q) * kTile + r0 + tx];
-        if (diag) {                                        // X^T: column r0 + tx holds this row's entries together
-            const float4* yr = reinterpret_cast<const float4*>(v + (r0 + tx) * kTile + c0);
-            const float4 y0 = yr[0], y1 = yr[1];
-            const float2 y[4] = {make_float2(y0.x, y0.y), make_float2(y0.z, y0.w), make_float2(y1.x, y1.y),
-                                 make_float2(y1.z, y1.w)};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int k = er + ex[kTile + c0 + q];
-                s[q] += scaled_double(x[q].x, k);
-                s[q] += scaled_double(y[q].x, k);
-                s[q] += scaled_double(__fadd_rn(x[q].y, y[q].y), k);   // parts below 2^-24 of the sums
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int k = er + ex[kTile + c0 + q];
-                s[q] += scaled_double(x[q].x, k);
-                s[q] += scaled_double(x[q].y, k);
-            }
+        for (int q = 0; q < 4; ++q) {
+            const int k = er + ex[kTile + c0 + q];
+            s[q] += scaled_double(x[q].x, k);
+            s[q] += scaled_double(x[q].y, k);
         }
     }
 #pragma unroll
@@ -592,32 +565,37 @@ int device_sms() {
     return sms;
 }
 
-// Row splits: about one CTA an SM, a tile of the diagonal 5/8 of the splits of the others (16 of 28 MMAs, the
-// fetches the same), at least 64 rows a split.
+// Row splits, the same for every tile: the count with the shortest schedule of at most three CTAs an SM, at
+// least 64 rows a split. In quarters of the time of a tile above the diagonal (0.124 us a row), one on the
+// diagonal takes three (0.094 us: its converters have half the work, the MMAs and fetches are the same), and
+// starting and ending a CTA about 260 rows. CTAs start in the order of their index, the long ones first. At
+// 1e6 x 256 that is 152 splits, every SM with one tile above and two on the diagonal (2.05 ms; 2.46 with 76
+// splits, 2.39 with 50 in one wave).
 GramPlan make_plan(int64_t m, int64_t d) {
-    const int64_t max_units = device_sms();
+    const int64_t sms = device_sms();
     GramPlan p;
     p.nt = (int)((d + kTile - 1) / kTile);
     p.noff = p.nt * (p.nt - 1) / 2;
-    const int64_t most = std::max<int64_t>(1, (m + 63) / 64);
-    int64_t so = 1, sd = 1;
-    for (int64_t k = 1; k <= 8 * most; ++k) {               // k / 8 splits of a tile above the diagonal
-        const int64_t o = std::min(most, std::max<int64_t>(1, k / 8)), q = std::min(most, std::max<int64_t>(1, (k * 5 + 32) / 64));
-        if (p.noff * o + p.nt * q > max_units) break;
-        so = o;
-        sd = q;
+    const int64_t most = std::max<int64_t>(1, std::min((m + 63) / 64, 3 * sms / (p.noff + p.nt)));
+    auto rows = [&](int64_t s) { return ((m + s - 1) / s + 15) / 16 * 16; };
+    int64_t best = INT64_MAX;
+    p.splits = 1;
+    for (int64_t s = 1; s <= most; ++s) {
+        const int64_t off = p.noff * s, dia = p.nt * s;
+        // the SMs end the long units at `t0` (`late` of them at t0 + 4); time for the others after that
+        const int64_t t0 = off / sms * 4, late = off % sms;
+        int64_t t = late ? 4 : 0;
+        while (late * ((t >= 4 ? t - 4 : 0) / 3) + (sms - late) * (t / 3) < dia) ++t;
+        const int64_t cost = (t0 + t) * rows(s) + 260 * ((off + dia + sms - 1) / sms);
+        if (cost < best) {
+            best = cost;
+            p.splits = (int)s;
+        }
     }
-    auto rows = [&](int64_t s) { return (int)(((m + s - 1) / s + 15) / 16 * 16); };
-    auto chunk = [&](int r) {
-        const int n = (r + kMaxChunk - 1) / kMaxChunk;
-        return std::min(kMaxChunk, ((r + n - 1) / n + 15) / 16 * 16);
-    };
-    p.rows_o = rows(so);
-    p.rows_d = rows(sd);
-    p.so = (int)std::max<int64_t>(1, (m + p.rows_o - 1) / p.rows_o);
-    p.sd = (int)std::max<int64_t>(1, (m + p.rows_d - 1) / p.rows_d);
-    p.chunk_o = chunk(p.rows_o);
-    p.chunk_d = chunk(p.rows_d);
+    p.rows = (int)rows(p.splits);
+    p.splits = (int)std::max<int64_t>(1, (m + p.rows - 1) / p.rows);
+    const int n = (p.rows + kMaxChunk - 1) / kMaxChunk;
+    p.chunk = std::min(kMaxChunk, ((p.rows + n - 1) / n + 15) / 16 * 16);
     return p;
 }
 
@@ -627,7 +605,7 @@ size_t colmax_doubles(int64_t m, int64_t d) { return (size_t)(((m + kMaxRows - 1
 
 size_t gram_tc_partial_doubles(int64_t m, int64_t d) {
     const GramPlan p = make_plan(m, d);
-    return (size_t)(p.noff * p.so + p.nt * p.sd) * kUnitDoubles + colmax_doubles(m, d);
+    return (size_t)(p.noff + p.nt) * p.splits * kUnitDoubles + colmax_doubles(m, d);
 }
 
 cudaError_t launch_gram_tc(const float* A, int64_t lda, int64_t m, int64_t d, double* Gp, double* G, int32_t* status,
@@ -636,7 +614,7 @@ cudaError_t launch_gram_tc(const float* A, int64_t lda, int64_t m, int64_t d, do
     const size_t smem = 1024 + (size_t)kStages * kStageBytes + kRingBytes + sizeof(GramCtl);
     cudaError_t e = cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const unsigned units = (unsigned)(p.noff * p.so + p.nt * p.sd);
+    const unsigned units = (unsigned)((p.noff + p.nt) * p.splits);
     uint32_t* colmax = reinterpret_cast<uint32_t*>(Gp + (size_t)units * kUnitDoubles);
     k_gram_colmax<<<dim3((unsigned)((m + kMaxRows - 1) / kMaxRows), (unsigned)p.nt), 512, 0, st>>>(A, lda, m, (int)d, colmax);
     k_gram_tc<<<units, kThreads, smem, st>>>(A, lda, m, (int)d, p, colmax, Gp, status);

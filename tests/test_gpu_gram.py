@@ -73,3 +73,18 @@ def test_gram_of_strided_rows(L, h, lda):
     want = torch.empty_like(theta)
     assert L.lev_exact_reference_dense(h, buf[:, :d], 1e-5, theta) == L.lev_exact_reference_dense(h, to_dev(A), 1e-5, want)
     np.testing.assert_allclose(to_np(theta), to_np(want), rtol=1e-5)
+
+
+@pytest.mark.parametrize("m,d", [(2055, 1023), (4100, 258), (40000, 100)])
+def test_equal_columns_tie(L, h, m, d):
+    """Twin columns lie in tiles on and above the diagonal; their entries of G are the same numbers, so the
+    lower index of each pair is the pivot and the rank is the number of pairs (and the odd column)."""
+    import torch
+    A = np.random.default_rng(d).standard_normal((m, d)).astype(np.float32)
+    A[:, d - d // 2:] = A[:, :d // 2]
+    perm = torch.empty(d, dtype=torch.int32, device="cuda")
+    R = torch.empty((d, d), dtype=torch.float64, device="cuda")
+    r = L.lev_rrqr(h, to_dev(A), 1e-4, perm, R)
+    assert L.lev_device_status(h) == 0
+    assert r == d - d // 2
+    assert to_np(perm)[:r].max() < r
