@@ -8,9 +8,10 @@
 // Dense: 128-row (64 for small n) x 256-column register tile, 16 x 8 per
 // thread, A and Mfull staged through shared memory in 16-wide k slices (two
 // stages), packed FP32 FMAs on row pairs.
-// CSR: one warp per row (product form of Lemma 1): the warp broadcasts each
-// (col, val) of the row and every lane accumulates 8 columns of
-// val * Mfull[col, :] with 128-bit loads; then squares and warp-sums.
+// CSR, long rows: one warp per row (product form of Lemma 1): the warp broadcasts
+// each (col, val) of the row and every lane accumulates 8 columns of
+// val * Mfull[col, :] with 128-bit loads; then squares and warp-sums. Short rows:
+// the pairs of the row's entries against P = Mfull Mfull^T.
 #include "f32x2.cuh"
 #include "lev_common.cuh"
 #include "lev_kernels.cuh"
@@ -257,112 +258,177 @@ __device__ __forceinline__ void df_term(float a, float b, float w, float2 P, flo
     tl = __fmaf_rn(xwe, P.x, tl);
 }
 
-// Rows with LO < len <= SEG entries (an empty row gets 0): SEG lanes a row, 32 / SEG rows a warp (a row is a short chain of
-// dependent loads, bounds then entries then P, so a warp keeps several in flight, the next rows'
-// bounds loaded ahead). Lane l of a row holds entry l; in step q the row's entry q is broadcast and
-// lane p <= q adds the pair (p, q), so each pair is taken once; the lanes' pairs are summed by
-// shuffles (TwoSum) at the end.
-template <int SEG, int LO>
+// Streaming loads of a row's entries: they are read once, so L1 keeps P.
+__device__ __forceinline__ int32_t ld_once(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_once(const float* p) {
+    float v;
+    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
+// The rows of `rows` (bit b: row r0 + b of the warp's 32, each of at most SEG entries; lane b holds its start p0
+// and length len), 32 / SEG at a time, SEG lanes a row, the next rows' entries loaded ahead. Lane l of a row
+// holds entry l; in step s it takes the pair (l, l + s mod len), so that len / 2 steps visit every pair of two
+// entries once with all lanes of the row at work (in the last step of an even length half of them). The
+// diagonal terms read dg (P's diagonal, shared memory). Four steps' reads of P are in flight together; their
+// terms are formed and summed two at a time with packed instructions, unweighted: the sum over p < q is doubled
+// once (exact) before the diagonal terms join it. A product's rounding error is taken against neg2 of the
+// rounded product: against a second product with a negated factor the results lost their low parts (2^-25 off).
+template <int SEG>
+__device__ __forceinline__ void csr_pair_rows(unsigned rows, int64_t p0, int len, int64_t r0, int lane,
+                                              const int32_t* __restrict__ col, const float* __restrict__ val, int d,
+                                              const float2* __restrict__ P, const float2* dg,
+                                              float* __restrict__ theta) {
+    if (!rows) return;
+    constexpr int RPW = 32 / SEG;
+    const int seg = lane / SEG, sl = lane % SEG;
+    int b, L, c;
+    float a;
+    auto fetch = [&]() {
+        b = -1;
+#pragma unroll
+        for (int g = 0; g < RPW; ++g) {
+            const int t = __ffs(rows) - 1;
+            rows &= rows - 1;
+            if (g == seg) b = t;
+        }
+        const int64_t at = __shfl_sync(0xffffffffu, p0, b & 31);
+        L = __shfl_sync(0xffffffffu, len, b & 31);
+        if (b < 0) L = 0;
+        c = -1;
+        a = 0.f;
+        if (sl < L) {
+            c = ld_once(col + at + sl);
+            a = ld_once(val + at + sl);
+        }
+    };
+    fetch();
+    for (bool more = true; more;) {
+        const int rb = b, Lc = L;
+        const bool in = (unsigned)c < (unsigned)d;
+        const int cp = in ? c : -1;
+        const float ap = in ? a : 0.f;
+        more = rows != 0;
+        if (more) fetch();
+        const int half = Lc >> 1;
+        // steps this lane takes: the last one of an even length belongs to the lower half of the lanes
+        const int mine = !in ? 0 : ((Lc & 1) == 0 && sl >= half ? half - 1 : half);
+        const int steps = RPW > 1 ? (int)__reduce_max_sync(0xffffffffu, (unsigned)half) : half;
+        const float2* Prow = P + (in ? cp * d : 0);
+        const f32x2 a2 = pack2(ap, ap);
+        f32x2 sh = 0ull, se = 0ull;
+        for (int s0 = 1; s0 <= steps; s0 += 4) {
+            float2 Pq[4];
+            float aq[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                int t = sl + s0 + u;
+                t -= t >= Lc ? Lc : 0;
+                const int src = lane - sl + (t & (SEG - 1));
+                const int cq = __shfl_sync(0xffffffffu, cp, src);
+                const float x = __shfl_sync(0xffffffffu, ap, src);
+                const bool ok = s0 + u <= mine && cq >= 0;
+                Pq[u] = make_float2(0.f, 0.f);
+                if (ok) Pq[u] = __ldg(Prow + cq);
+                aq[u] = ok ? x : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u += 2) {
+                const f32x2 q = pack2(aq[u], aq[u + 1]);
+                const f32x2 hi = pack2(Pq[u].x, Pq[u + 1].x), lo = pack2(Pq[u].y, Pq[u + 1].y);
+                const f32x2 x = mul2(a2, q);
+                const f32x2 xe = fma2(a2, q, neg2(x));                // a_p a_q = x + xe exactly
+                const f32x2 th = mul2(x, hi);
+                f32x2 tl = fma2(x, hi, neg2(th));
+                tl = fma2(x, lo, tl);
+                tl = fma2(xe, hi, tl);
+                const f32x2 sum = add2(sh, th);                       // TwoSum; the remainders collect in se
+                const f32x2 bb = sub2(sum, sh);
+                const f32x2 er = add2(sub2(sh, sub2(sum, bb)), sub2(th, bb));
+                se = add2(se, add2(er, tl));
+                sh = sum;
+            }
+        }
+        float h0, h1, e0, e1;
+        unpack2(sh, h0, h1);
+        unpack2(se, e0, e1);
+        df_add(h0, e0, h1, e1);
+        h0 = __fmul_rn(h0, 2.f);
+        e0 = __fmul_rn(e0, 2.f);
+        float dh = 0.f, dl = 0.f;
+        if (in) df_term(ap, ap, 1.f, dg[cp], dh, dl);
+        df_add(h0, e0, dh, dl);
+#pragma unroll
+        for (int o = SEG / 2; o > 0; o >>= 1) {
+            const float oh = __shfl_xor_sync(0xffffffffu, h0, o), oe = __shfl_xor_sync(0xffffffffu, e0, o);
+            df_add(h0, e0, oh, oe);
+        }
+        if (sl == 0 && rb >= 0) theta[r0 + rb] = __fadd_rn(h0, e0);
+    }
+}
+
+// Every row of at most 32 entries by the second form (an empty row gets 0): a warp reads the bounds of 32 rows
+// at once (the next 32 loaded ahead) and takes them by class, 8, 16 or 32 lanes a row. Bound by L1 at 89%: each
+// read of P is a line of its own (P is 8 MB at d = 1,024, 2% of the reads hit), so len (len - 1) / 2 reads a row
+// with the diagonal in shared memory instead of len (len + 1) / 2, and one pass over the bounds instead of one
+// for each class, are what counts. 8e7 rows of 12 entries, d = 1,024: 29.3 -> 20.0 ms with k_final_csr_long
+// (a lane took the pairs (p, q >= p), one read in flight a warp); 8e6 rows of 8 with 1% of 256: 2.9 -> 2.1 ms.
 __global__ void __launch_bounds__(256) k_final_csr_pairs(const int64_t* __restrict__ row_ptr,
                                                          const int32_t* __restrict__ col,
                                                          const float* __restrict__ val, int64_t n, int d,
                                                          const float2* __restrict__ P, float* __restrict__ theta) {
-    constexpr int RPW = 32 / SEG;
-    const int lane = threadIdx.x & 31, seg = lane / SEG, sl = lane % SEG;
+    __shared__ float2 dg[1024];
+    for (int j = threadIdx.x; j < d; j += blockDim.x) dg[j] = P[(int64_t)j * (d + 1)];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    int64_t rn = warp * RPW + seg;
-    int64_t np0 = rn < n ? row_ptr[rn] : 0, np1 = rn < n ? row_ptr[rn + 1] : 0;
-    for (int64_t r0 = warp * RPW; r0 < n; r0 += nwarps * RPW) {
-        const int64_t r = r0 + seg;
-        const int64_t p0 = np0, p1 = np1;
-        const int len = (int)(p1 - p0);
-        const bool mine = r < n && len > LO && len <= SEG;
-        int c = -1;
-        float a = 0.f;
-        if (mine && sl < len) {
-            c = col[p0 + sl];
-            a = val[p0 + sl];
-        }
-        rn = r + nwarps * RPW;
+    int64_t rn = warp * 32 + lane;
+    int64_t np0 = rn < n ? row_ptr[rn] : 0, np1 = rn < n ? row_ptr[rn + 1] : -1;
+    for (int64_t r0 = warp * 32; r0 < n; r0 += nwarps * 32) {
+        const int64_t p0 = np0, len64 = np1 - np0;                    // past the end: length -1, in no class
+        rn += nwarps * 32;
         np0 = rn < n ? row_ptr[rn] : 0;
-        np1 = rn < n ? row_ptr[rn + 1] : 0;
-        if ((unsigned)c >= (unsigned)d) { c = -1; a = 0.f; }
-        const int len_w = mine ? len : 0;
-        int steps = len_w;                                            // the longest row of the warp
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) steps = max(steps, __shfl_xor_sync(0xffffffffu, steps, o));
-        float sh = 0.f, sl2 = 0.f;
-        const int64_t prow = c >= 0 ? (int64_t)c * d : 0;
-        for (int q = 0; q < steps; ++q) {
-            const int cq = __shfl_sync(0xffffffffu, c, seg * SEG + q);
-            const float aq = __shfl_sync(0xffffffffu, a, seg * SEG + q);
-            if (q < len_w && sl <= q && c >= 0 && cq >= 0) {
-                float th, tl;
-                df_term(a, aq, sl == q ? 1.f : 2.f, P[prow + cq], th, tl);
-                df_add(sh, sl2, th, tl);
-            }
-        }
-#pragma unroll
-        for (int o = SEG / 2; o > 0; o >>= 1) {
-            const float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sl2, o);
-            df_add(sh, sl2, oh, ol);
-        }
-        if (mine && sl == 0) theta[r] = __fadd_rn(sh, sl2);
+        np1 = rn < n ? row_ptr[rn + 1] : -1;
+        const int len = (int)min(len64, (int64_t)64);
+        const unsigned m8 = __ballot_sync(0xffffffffu, len64 >= 0 && len64 <= 8);
+        const unsigned m16 = __ballot_sync(0xffffffffu, len64 > 8 && len64 <= 16);
+        const unsigned m32 = __ballot_sync(0xffffffffu, len64 > 16 && len64 <= 32);
+        csr_pair_rows<8>(m8, p0, len, r0, lane, col, val, d, P, dg, theta);
+        csr_pair_rows<16>(m16, p0, len, r0, lane, col, val, d, P, dg, theta);
+        csr_pair_rows<32>(m32, p0, len, r0, lane, col, val, d, P, dg, theta);
     }
 }
 
-// Rows of more than 16 entries: a warp scans the bounds of 32 rows at once and takes each such row
-// in turn with the whole warp: the second form (one entry per lane, the pair loop above) up to 32
-// entries, the first form (csr_row_norm) above.
+// Rows of more than 32 entries by the first form: a warp scans the bounds of 32 rows at once (the next 32
+// loaded ahead) and takes each such row in turn.
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_final_csr_long(const int64_t* __restrict__ row_ptr,
                                                         const int32_t* __restrict__ col,
                                                         const float* __restrict__ val, int64_t n, int d,
                                                         const float* __restrict__ M, int k,
-                                                        const float2* __restrict__ P, float* __restrict__ theta) {
+                                                        float* __restrict__ theta) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    int64_t rn = warp * 32 + lane;
+    int64_t np0 = rn < n ? row_ptr[rn] : 0, np1 = rn < n ? row_ptr[rn + 1] : 0;
     for (int64_t r0 = warp * 32; r0 < n; r0 += nwarps * 32) {
-        const int64_t rl = r0 + lane;
-        const int64_t lenl = rl < n ? row_ptr[rl + 1] - row_ptr[rl] : 0;
-        unsigned todo = __ballot_sync(0xffffffffu, lenl > 16);
+        const int64_t b0 = np0, b1 = np1;
+        rn += nwarps * 32;
+        np0 = rn < n ? row_ptr[rn] : 0;
+        np1 = rn < n ? row_ptr[rn + 1] : 0;
+        unsigned todo = __ballot_sync(0xffffffffu, b1 - b0 > 32);
         while (todo) {
             const int b = __ffs(todo) - 1;
             todo &= todo - 1;
-            const int64_t i = r0 + b;
-            const int64_t p0 = row_ptr[i], p1 = row_ptr[i + 1];
-            const int len = (int)(p1 - p0);
-            if (len > 32) {
-                const float total = warp_sum(csr_row_norm<VEC>(p0, p1, col, val, d, M, k, lane));
-                if (lane == 0) theta[i] = total;
-                continue;
-            }
-            int c = -1;
-            float a = 0.f;
-            if (lane < len) {
-                c = col[p0 + lane];
-                a = val[p0 + lane];
-                if ((unsigned)c >= (unsigned)d) { c = -1; a = 0.f; }
-            }
-            float sh = 0.f, sl2 = 0.f;
-            const int64_t prow = c >= 0 ? (int64_t)c * d : 0;
-            for (int q = 0; q < len; ++q) {
-                const int cq = __shfl_sync(0xffffffffu, c, q);
-                const float aq = __shfl_sync(0xffffffffu, a, q);
-                if (lane <= q && c >= 0 && cq >= 0) {
-                    float th, tl;
-                    df_term(a, aq, lane == q ? 1.f : 2.f, P[prow + cq], th, tl);
-                    df_add(sh, sl2, th, tl);
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sl2, o);
-                df_add(sh, sl2, oh, ol);
-            }
-            if (lane == 0) theta[i] = __fadd_rn(sh, sl2);
+            const int64_t p0 = __shfl_sync(0xffffffffu, b0, b), p1 = __shfl_sync(0xffffffffu, b1, b);
+            const float total = warp_sum(csr_row_norm<VEC>(p0, p1, col, val, d, M, k, lane));
+            if (lane == 0) theta[r0 + b] = total;
         }
     }
 }
@@ -430,23 +496,17 @@ cudaError_t launch_final_csr_gram(const int64_t* row_ptr, const int32_t* col, co
     if (e != cudaSuccess) return e;
     k_split_pairs<<<152 * 4, 256, 0, st>>>(P, d * d, Pdf);
     const bool vec = (reinterpret_cast<uintptr_t>(Mfull) % 16 == 0) && (k % 4 == 0);
-    int64_t grid = (n * 8 + 255) / 256;                 // four rows of up to 8 entries a warp
-    if (grid > 152 * 64) grid = 152 * 64;
+    int64_t grid = (n + 255) / 256;                     // 32 rows a warp at a time
+    if (grid > 152 * 24) grid = 152 * 24;
     if (grid < 1) grid = 1;
-    k_final_csr_pairs<8, -1><<<(unsigned)grid, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Pdf, theta);  // empty rows too
-    int64_t grid16 = (n * 16 + 255) / 256;              // two rows of 9 to 16 entries a warp
-    if (grid16 > 152 * 64) grid16 = 152 * 64;
-    if (grid16 < 1) grid16 = 1;
-    k_final_csr_pairs<16, 8><<<(unsigned)grid16, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Pdf, theta);
+    k_final_csr_pairs<<<(unsigned)grid, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Pdf, theta);  // empty rows too
     int64_t grid_l = (n + 255) / 256;                   // 32 rows scanned a warp
     if (grid_l > 152 * 16) grid_l = 152 * 16;
     if (grid_l < 1) grid_l = 1;
     if (vec)
-        k_final_csr_long<true><<<(unsigned)grid_l, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Mfull, (int)k, Pdf,
-                                                                theta);
+        k_final_csr_long<true><<<(unsigned)grid_l, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Mfull, (int)k, theta);
     else
-        k_final_csr_long<false><<<(unsigned)grid_l, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Mfull, (int)k, Pdf,
-                                                                 theta);
+        k_final_csr_long<false><<<(unsigned)grid_l, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Mfull, (int)k, theta);
     return cudaGetLastError();
 }
 
