@@ -2,6 +2,8 @@
 // the right factor (qr.cu).
 #pragma once
 
+#include "f32x2.cuh"
+
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -37,6 +39,19 @@ __device__ __forceinline__ float2 df_sub_mul(float2 x, float2 a, float2 b) {
     err = __fadd_rn(err, __fsub_rn(x.y, pe));
     const float h = __fadd_rn(s, err);
     return make_float2(h, __fsub_rn(err, __fsub_rn(h, s)));
+}
+// x - a b on two packed double-floats, the operations of df_sub_mul in its order.
+__device__ __forceinline__ void df_sub_mul2(f32x2& xh, f32x2& xl, f32x2 ah, f32x2 al, f32x2 bh, f32x2 bl) {
+    const f32x2 p = mul2(ah, bh);
+    f32x2 pe = fma2(ah, bh, neg2(p));
+    pe = fma2(ah, bl, pe);
+    pe = fma2(al, bh, pe);
+    const f32x2 s = sub2(xh, p), bb = sub2(s, xh);
+    f32x2 err = add2(sub2(xh, sub2(s, bb)), sub2(neg2(p), bb));
+    err = add2(err, sub2(xl, pe));
+    const f32x2 h = add2(s, err);
+    xl = sub2(err, sub2(h, s));
+    xh = h;
 }
 // 1 / sqrt(v) for a positive double-float v: an FP32 estimate, one FP32 Newton step, then one step
 // y + y (1 - v y^2) / 2 with the residual formed in double-float (to about 2^-46)

@@ -518,19 +518,6 @@ __global__ void __launch_bounds__(NT, 1) k_pchol_grid(const double* __restrict__
     if (me == 0 && tid == 0) *rank_out = j;
 }
 
-// x - a b on two packed double-floats, the operations of df_sub_mul in its order.
-__device__ __forceinline__ void df_sub_mul2(f32x2& xh, f32x2& xl, f32x2 ah, f32x2 al, f32x2 bh, f32x2 bl) {
-    const f32x2 p = mul2(ah, bh);
-    f32x2 pe = fma2(ah, bh, neg2(p));
-    pe = fma2(ah, bl, pe);
-    pe = fma2(al, bh, pe);
-    const f32x2 s = sub2(xh, p), bb = sub2(s, xh);
-    f32x2 err = add2(sub2(xh, sub2(s, bb)), sub2(neg2(p), bb));
-    err = add2(err, sub2(xl, pe));
-    const f32x2 h = add2(s, err);
-    xl = sub2(err, sub2(h, s));
-    xh = h;
-}
 // The FP32 value an order_key32 was made from.
 __device__ __forceinline__ float key32_value(unsigned k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);

@@ -324,53 +324,121 @@ __global__ void k_scaled_transpose_df(const double* __restrict__ R, const int64_
     }
 }
 
-// M = R_11^{-1} Omega column by column, one CTA per column q and one thread per row i (r <= 1024),
-// in double-float arithmetic (FP32 pairs, about 48 bits; FP64 runs at 1/64 of the FP32 rate on
-// GB300 and bound this solve at d = 1,024): with the unit-diagonal form
-// x_i = w_i / R_ii - sum_{j > i} (R_ij / R_ii) x_j, step j (from the bottom) publishes x_j through
-// shared memory (double-buffered by step parity, one barrier per step) and every thread i < j
-// subtracts Rs[j][i] x_j, so each row sees its updates in the order j = r-1, ..., i+1. The
-// coefficients of the next eight steps are loaded ahead. Row i of M goes to row perm[i] of Mfull,
-// rounded to FP32.
+// M = R_11^{-1} Omega, one CTA per two columns q, q + 1 and one thread per row i (r <= 1024), in
+// double-float arithmetic (FP32 pairs, about 48 bits; FP64 runs at 1/64 of the FP32 rate on GB300),
+// the two columns packed in one instruction: with the unit-diagonal form
+// x_i = w_i / R_ii - sum_{j > i} (R_ij / R_ii) x_j, each row takes its updates in the order
+// j = r-1, ..., i+1. Bound by the chain of those updates: with one row published a barrier it was
+// 0.42 us a row at r = 1,024. Rows therefore go in blocks of 32, a warp a block: the warp solves its
+// block by shuffles, publishes the 32 solutions (double-buffered by block parity, one barrier a
+// block), and the warps of the rows above subtract them while the next warp, done with its own,
+// solves its block. The coefficients come ahead by cp.async, whose groups are waited for in order
+// (registers loaded eight rows ahead shared scoreboards and waited for the youngest load, 300 cycles
+// a row). Row i of M goes to row perm[i] of
+// Mfull, rounded to FP32. Identity right-hand sides (R^{-1}) start at the block of their own row: the
+// rows below it are 0; the longest columns go first.
 // With the factor Lc of Omega's Gram matrix (upper U, row q holding column q of L = U^T) and
-// r < k, r <= *d_kc, the right-hand side is column q of L_r instead and the CTAs q >= r leave
-// their column 0.
-constexpr int OMEGA_PF = 8;
+// r < k, r <= *d_kc, the right-hand side is column q of L_r instead and the columns q >= r stay 0.
+// us, with one CTA a column and a barrier a row before: d = k = 1,024 identity 1380 -> 375; d = 1,024,
+// k = 256 430 -> 228; r = 200, k = 256 41 -> 36.
+constexpr int OMEGA_CH = 8, OMEGA_ST = 3;                     // rows a chunk, chunks in flight
 __global__ void __launch_bounds__(1024) k_omega_solve(const double* __restrict__ R, const float2* __restrict__ Rs,
                                                       const double* __restrict__ Om, const double* __restrict__ Lc,
                                                       int kc, const int64_t* __restrict__ d_kc,
                                                       const int32_t* __restrict__ perm,
                                                       const int64_t* __restrict__ d_rank, int d, int k, int identity,
                                                       float* __restrict__ Mfull) {
-    __shared__ float2 xs[2];
-    const int q = blockIdx.x, i = threadIdx.x;
+    extern __shared__ float2 coefs[];                            // [warp][OMEGA_ST][OMEGA_CH][32]
+    __shared__ ulonglong2 xs[2][32];                             // {high, low} parts of both columns
+    const int i = threadIdx.x, lane = i & 31, w = i >> 5;
+    const int q0 = 2 * (int)(gridDim.x - 1 - blockIdx.x);
     const int r = (int)min(max(*d_rank, (int64_t)0), (int64_t)d);
     const bool reduced = Lc != nullptr && !identity && r < k && r <= kc && (int64_t)r <= *d_kc;
-    if (reduced && q >= r) return;                               // the whole CTA: Mfull column q stays 0
-    float2 x = make_float2(0.f, 0.f);
+    // columns of this CTA that are not 0 (the whole CTA leaves when there are none)
+    const int ncol = min((reduced || identity) ? min(r, k) : k, q0 + 2) - q0;
+    if (ncol <= 0 || r == 0) return;
+    float2 x0 = make_float2(0.f, 0.f), x1 = x0;
     if (i < r) {
-        const double w = identity ? (i == q ? 1.0 : 0.0)
-                                  : (reduced ? Lc[(int64_t)q * kc + i] : Om[(int64_t)i * k + q]);
-        x = df_from_double(w / R[(int64_t)i * d + i]);
+        const double rii = R[(int64_t)i * d + i];
+        auto rhs = [&](int q) {
+            return df_from_double((identity ? (i == q ? 1.0 : 0.0)
+                                            : (reduced ? Lc[(int64_t)q * kc + i] : Om[(int64_t)i * k + q])) / rii);
+        };
+        x0 = rhs(q0);
+        if (ncol > 1) x1 = rhs(q0 + 1);
     }
-    // ring of coefficients: c[t] holds Rs[j - t][i] for the current step j
-    float2 c[OMEGA_PF];
+    f32x2 xh = pack2(x0.x, x1.x), xl = pack2(x0.y, x1.y);
+    auto subtract = [&](float2 c, f32x2 bh, f32x2 bl) {
+        df_sub_mul2(xh, xl, pack2(c.x, c.x), pack2(c.y, c.y), bh, bl);
+    };
+    // The coefficients Rs[j][i] of this thread, j descending from the top block to its own, by chunks of 8
+    // rows through OMEGA_ST stages; 0 outside the strict triangle and past the rank. A thread reads only what
+    // it copied itself.
+    const int Jt = (identity ? q0 + ncol - 1 : r - 1) >> 5;
+    float2* ring = coefs + (size_t)w * (OMEGA_ST * OMEGA_CH * 32) + lane;
+    int next = Jt * 32 + 31, slot_in = 0, slot = 0;
+    auto copy_chunk = [&]() {
+        if (next >= w * 32) {
+            const unsigned to = (unsigned)__cvta_generic_to_shared(ring + slot_in * (OMEGA_CH * 32));
 #pragma unroll
-    for (int t = 0; t < OMEGA_PF; ++t) {
-        const int j = r - 1 - t;
-        c[t] = (j > i) ? Rs[(int64_t)j * d + i] : make_float2(0.f, 0.f);
-    }
-    for (int j = r - 1; j >= 0; --j) {
-        const float2 cj = c[0];
+            for (int u = 0; u < OMEGA_CH; ++u) {
+                const int j = next - u;
+                const bool ok = j > i && j < r;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;"
+                             :: "r"(to + u * 256), "l"(ok ? Rs + (int64_t)j * d + i : Rs), "r"(ok ? 8 : 0) : "memory");
+            }
+            next -= OMEGA_CH;
+            slot_in = slot_in + 1 == OMEGA_ST ? 0 : slot_in + 1;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // the next chunk's coefficients; the chunk after those in flight is asked for
+    auto chunk = [&](float2* c) {
+        copy_chunk();
+        asm volatile("cp.async.wait_group %0;" :: "n"(OMEGA_ST - 1) : "memory");
 #pragma unroll
-        for (int t = 0; t + 1 < OMEGA_PF; ++t) c[t] = c[t + 1];
-        const int jn = j - OMEGA_PF;
-        c[OMEGA_PF - 1] = (jn > i) ? Rs[(int64_t)jn * d + i] : make_float2(0.f, 0.f);
-        if (i == j) xs[j & 1] = x;
+        for (int u = 0; u < OMEGA_CH; ++u) c[u] = ring[slot * (OMEGA_CH * 32) + u * 32];
+        slot = slot + 1 == OMEGA_ST ? 0 : slot + 1;
+    };
+#pragma unroll
+    for (int t = 0; t + 1 < OMEGA_ST; ++t) copy_chunk();
+    for (int J = Jt; J >= 0; --J) {
+        ulonglong2* buf = xs[J & 1];
+        float2 c[OMEGA_CH];
+        if (w == J) {
+#pragma unroll 1
+            for (int tb = 31; tb >= 0; tb -= OMEGA_CH) {
+                chunk(c);
+#pragma unroll
+                for (int u = 0; u < OMEGA_CH; ++u) {
+                    const int t = tb - u;
+                    const f32x2 bh = __shfl_sync(0xffffffffu, xh, t), bl = __shfl_sync(0xffffffffu, xl, t);
+                    if (lane < t) subtract(c[u], bh, bl);
+                }
+            }
+            buf[lane] = make_ulonglong2(xh, xl);
+        }
         __syncthreads();
-        if (i < j) x = df_sub_mul(x, cj, xs[j & 1]);
+        if (w < J) {
+#pragma unroll 1
+            for (int tb = 31; tb >= 0; tb -= OMEGA_CH) {
+                chunk(c);
+#pragma unroll
+                for (int u = 0; u < OMEGA_CH; ++u) {
+                    const ulonglong2 b = buf[tb - u];
+                    subtract(c[u], b.x, b.y);
+                }
+            }
+        }
     }
-    if (i < r) Mfull[(int64_t)perm[i] * k + q] = (float)df_to_double(x);
+    if (i < r) {
+        float h0, h1, l0, l1;
+        unpack2(xh, h0, h1);
+        unpack2(xl, l0, l1);
+        float* out = Mfull + (int64_t)perm[i] * k + q0;
+        out[0] = (float)df_to_double(make_float2(h0, l0));
+        if (ncol > 1) out[1] = (float)df_to_double(make_float2(h1, l1));
+    }
 }
 
 }  // namespace
@@ -501,7 +569,11 @@ cudaError_t launch_omega_factor(const double* R, const int32_t* perm, const int6
         float2* Rs2 = reinterpret_cast<float2*>(Rs);                // the same d x d bytes
         k_scaled_transpose_df<<<grid, 256, 0, st>>>(R, d_rank, (int)d, Rs2);
         const int threads = (int)((d + 31) / 32 * 32);
-        k_omega_solve<<<(unsigned)k, threads, 0, st>>>(R, Rs2, Omega, Lc && d_kc ? Lc : nullptr, (int)kc, d_kc,
+        const size_t smem = sizeof(float2) * (size_t)threads * OMEGA_CH * OMEGA_ST;
+        e = cudaFuncSetAttribute(k_omega_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(float2) * 1024 * OMEGA_CH * OMEGA_ST);
+        if (e != cudaSuccess) return e;
+        k_omega_solve<<<(unsigned)((k + 1) / 2), threads, smem, st>>>(R, Rs2, Omega, Lc && d_kc ? Lc : nullptr, (int)kc, d_kc,
                                                        perm, d_rank, (int)d, (int)k, omega_identity ? 1 : 0, Mfull);
         return cudaGetLastError();
     }
