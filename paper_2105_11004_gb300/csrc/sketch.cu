@@ -12,6 +12,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "f32x2.cuh"
 #include "lev_common.cuh"
@@ -293,8 +294,25 @@ __global__ void __launch_bounds__(256) k_countsketch_dense_scalar(
 // at once (lane r holds row r's), and the first 32 entries of eight rows are
 // loaded before any of them is added, so the dependent global loads of a
 // bucket overlap instead of running one row at a time; entries past the 32nd
-// of a row (the heavy rows) follow in that row's turn.
+// of a row (the heavy rows) follow in that row's turn. What bounds it is the
+// rows' scattered sectors (about 290 bytes of DRAM a row of 12 entries) in
+// what L1 the accumulators leave: entries pass it by, so that a row's two
+// bounds meet there (44 warps an SM, with nearly no L1 left, took 11.5 ms).
+// A row costs four shuffles, and entries whose columns ascend strictly, as those
+// of sorted rows do, are added by plain loads and stores; other rows take
+// shared-memory atomics. 8e7 rows of 12 entries: 6.75 -> 6.38 ms; 2e6 of 8 and
+// 1% of 256: 253 -> 235 us.
 constexpr int CS_PF = 8;
+__device__ __forceinline__ int32_t ld_entry(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_entry(const float* p) {
+    float v;
+    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 // Bucket b added into the warp's zeroed accumulator row sacc (d floats).
 __device__ __forceinline__ void csr_bucket_sum(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                                const float* __restrict__ val, int d, const int* __restrict__ off,
@@ -303,38 +321,43 @@ __device__ __forceinline__ void csr_bucket_sum(const int64_t* __restrict__ row_p
     for (int tb = t0; tb < t1; tb += 32) {
         const int nr = min(32, t1 - tb);
         int64_t my_p0 = 0, my_p1 = 0;
-        float my_sg = 0.f;
+        int my_len = 0;                                      // min(length, 33), + 64 for the sign -
         if (lane < nr) {
             const uint32_t e = perm[tb + lane];
             const int64_t row = e & ~kSignBit;
-            my_sg = (e & kSignBit) ? -1.f : 1.f;
             my_p0 = row_ptr[row];
             my_p1 = row_ptr[row + 1];
+            my_len = (int)max((int64_t)0, min((int64_t)33, my_p1 - my_p0)) + ((e & kSignBit) ? 64 : 0);
         }
         for (int r0 = 0; r0 < nr; r0 += CS_PF) {
-            int cc[CS_PF];
+            int cc[CS_PF], ln[CS_PF];
             float vv[CS_PF];
 #pragma unroll
             for (int u = 0; u < CS_PF; ++u) {                // loads of CS_PF rows in flight together
-                const int r = r0 + u;
-                const int64_t p0 = __shfl_sync(0xffffffffu, my_p0, r & 31);
-                const int64_t p1 = __shfl_sync(0xffffffffu, my_p1, r & 31);
-                cc[u] = -1;
+                const int r = (r0 + u) & 31;                 // past nr: length 0
+                const int64_t p = __shfl_sync(0xffffffffu, my_p0, r) + lane;
+                ln[u] = __shfl_sync(0xffffffffu, my_len, r);
+                cc[u] = INT_MAX;
                 vv[u] = 0.f;
-                if (r < nr && p0 + lane < p1) {
-                    cc[u] = col[p0 + lane];
-                    vv[u] = val[p0 + lane];
+                if (lane < (ln[u] & 63)) {
+                    cc[u] = ld_entry(col + p);
+                    vv[u] = ld_entry(val + p);
                 }
             }
 #pragma unroll
             for (int u = 0; u < CS_PF; ++u) {                // rows added in order
-                const int r = r0 + u;
-                const int64_t p0 = __shfl_sync(0xffffffffu, my_p0, r & 31);
-                const int64_t p1 = __shfl_sync(0xffffffffu, my_p1, r & 31);
-                const float sg = __shfl_sync(0xffffffffu, my_sg, r & 31);
-                if (r < nr) {
-                    if ((unsigned)cc[u] < (unsigned)d) atomicAdd(&sacc[cc[u]], sg * vv[u]);
-                    for (int64_t p = p0 + 32 + lane; p < p1; p += 32) {
+                if (r0 + u >= nr) break;
+                const float sg = ln[u] & 64 ? -1.f : 1.f;
+                const int before = __shfl_up_sync(0xffffffffu, cc[u], 1);
+                const bool sorted = __all_sync(0xffffffffu, lane == 0 || before < cc[u] || cc[u] == INT_MAX);
+                if ((unsigned)cc[u] < (unsigned)d) {
+                    if (sorted) sacc[cc[u]] += sg * vv[u];
+                    else atomicAdd(&sacc[cc[u]], sg * vv[u]);
+                }
+                if ((ln[u] & 63) > 32) {
+                    __syncwarp();
+                    const int64_t p1 = __shfl_sync(0xffffffffu, my_p1, r0 + u);
+                    for (int64_t p = __shfl_sync(0xffffffffu, my_p0, r0 + u) + 32 + lane; p < p1; p += 32) {
                         const int c = col[p];
                         if ((unsigned)c < (unsigned)d) atomicAdd(&sacc[c], sg * val[p]);
                     }
@@ -345,22 +368,33 @@ __device__ __forceinline__ void csr_bucket_sum(const int64_t* __restrict__ row_p
     }
 }
 
+// V4: d is a multiple of 4 and B is 16-byte aligned.
+template <bool V4>
 __global__ void __launch_bounds__(128) k_countsketch_csr(
         const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
         const float* __restrict__ val, int d, const int* __restrict__ off,
         const uint32_t* __restrict__ perm, int s, float* __restrict__ B) {
-    extern __shared__ float sacc_all[];
+    extern __shared__ float4 sacc_all[];
     const int wib = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    float* sacc = sacc_all + (int64_t)wib * d;
+    float* sacc = reinterpret_cast<float*>(sacc_all) + (int64_t)wib * d;
     const int warp = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int nwarps = (int)((gridDim.x * (int64_t)blockDim.x) >> 5);
     for (int b = warp; b < s; b += nwarps) {
-        for (int c = lane; c < d; c += 32) sacc[c] = 0.f;
+        if (V4) {
+            for (int c = lane * 4; c < d; c += 128) *reinterpret_cast<float4*>(sacc + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+        } else {
+            for (int c = lane; c < d; c += 32) sacc[c] = 0.f;
+        }
         __syncwarp();
         csr_bucket_sum(row_ptr, col, val, d, off, perm, b, lane, sacc);
         float* out = B + (int64_t)b * d;
-        for (int c = lane; c < d; c += 32) out[c] = sacc[c];
+        if (V4) {
+            for (int c = lane * 4; c < d; c += 128)
+                *reinterpret_cast<float4*>(out + c) = *reinterpret_cast<const float4*>(sacc + c);
+        } else {
+            for (int c = lane; c < d; c += 32) out[c] = sacc[c];
+        }
         __syncwarp();
     }
 }
@@ -696,13 +730,13 @@ cudaError_t launch_countsketch_csr(const int64_t* row_ptr, const int32_t* col, c
                                    float* B, cudaStream_t st) {
     const int warps = 4;
     const size_t smem = sizeof(float) * (size_t)d * warps;
+    auto* kern = d % 4 == 0 && reinterpret_cast<uintptr_t>(B) % 16 == 0 ? k_countsketch_csr<true>
+                                                                        : k_countsketch_csr<false>;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_countsketch_csr,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_countsketch_csr<<<grid_for(s * 32, 32 * warps), 32 * warps, smem, st>>>(
-        row_ptr, col, val, (int)d, off, perm, (int)s, B);
+    kern<<<grid_for(s * 32, 32 * warps), 32 * warps, smem, st>>>(row_ptr, col, val, (int)d, off, perm, (int)s, B);
     return cudaGetLastError();
 }
 
