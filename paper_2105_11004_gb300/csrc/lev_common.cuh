@@ -101,7 +101,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned& epoch, i
         while (ld_acquire_gpu(count) < target) {
             if (ld_volatile(status) != 0) break;
             if (++spins > kSpinLimit) { atomicExch(status, kStatusTimeoutBarrier); break; }
-            __nanosleep(256);
+            if (spins > 128) __nanosleep(256);          // first polls without a pause: most waits are short
         }
         __threadfence();
     } else {
