@@ -372,15 +372,17 @@ __device__ __forceinline__ void csr_pair_rows(unsigned rows, int64_t p0, int len
 }
 
 // Every row of at most 32 entries by the second form (an empty row gets 0): a warp reads the bounds of 32 rows
-// at once (the next 32 loaded ahead) and takes them by class, 8, 16 or 32 lanes a row. Bound by L1 at 89%: each
+// at once (the next 32 loaded ahead), takes them by class, 8, 16 or 32 lanes a row, and notes whether any is
+// longer. Bound by L1 at 89%: each
 // read of P is a line of its own (P is 8 MB at d = 1,024, 2% of the reads hit), so len (len - 1) / 2 reads a row
 // with the diagonal in shared memory instead of len (len + 1) / 2, and one pass over the bounds instead of one
-// for each class, are what counts. 8e7 rows of 12 entries, d = 1,024: 29.3 -> 20.0 ms with k_final_csr_long
+// for each class, are what counts. 8e7 rows of 12 entries, d = 1,024: 29.3 -> 19.5 ms with k_final_csr_long
 // (a lane took the pairs (p, q >= p), one read in flight a warp); 8e6 rows of 8 with 1% of 256: 2.9 -> 2.1 ms.
 __global__ void __launch_bounds__(256) k_final_csr_pairs(const int64_t* __restrict__ row_ptr,
                                                          const int32_t* __restrict__ col,
                                                          const float* __restrict__ val, int64_t n, int d,
-                                                         const float2* __restrict__ P, float* __restrict__ theta) {
+                                                         const float2* __restrict__ P, int* __restrict__ longer_seen,
+                                                         float* __restrict__ theta) {
     __shared__ float2 dg[1024];
     for (int j = threadIdx.x; j < d; j += blockDim.x) dg[j] = P[(int64_t)j * (d + 1)];
     __syncthreads();
@@ -398,6 +400,7 @@ __global__ void __launch_bounds__(256) k_final_csr_pairs(const int64_t* __restri
         const unsigned m8 = __ballot_sync(0xffffffffu, len64 >= 0 && len64 <= 8);
         const unsigned m16 = __ballot_sync(0xffffffffu, len64 > 8 && len64 <= 16);
         const unsigned m32 = __ballot_sync(0xffffffffu, len64 > 16 && len64 <= 32);
+        if (__any_sync(0xffffffffu, len64 > 32) && lane == 0) *longer_seen = 1;
         csr_pair_rows<8>(m8, p0, len, r0, lane, col, val, d, P, dg, theta);
         csr_pair_rows<16>(m16, p0, len, r0, lane, col, val, d, P, dg, theta);
         csr_pair_rows<32>(m32, p0, len, r0, lane, col, val, d, P, dg, theta);
@@ -405,13 +408,16 @@ __global__ void __launch_bounds__(256) k_final_csr_pairs(const int64_t* __restri
 }
 
 // Rows of more than 32 entries by the first form: a warp scans the bounds of 32 rows at once (the next 32
-// loaded ahead) and takes each such row in turn.
+// loaded ahead) and takes each such row in turn; nothing to do when k_final_csr_pairs saw no such row (the scan
+// alone took 0.46 ms at 8e7 rows). Finding the rows by masks that the pairs' pass leaves, or scanning 128 bounds
+// at once, cost registers that the rows' own loop needs (1.46 against 1.30 ms at 8e4 rows of 256 entries).
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_final_csr_long(const int64_t* __restrict__ row_ptr,
                                                         const int32_t* __restrict__ col,
                                                         const float* __restrict__ val, int64_t n, int d,
                                                         const float* __restrict__ M, int k,
-                                                        float* __restrict__ theta) {
+                                                        const int* __restrict__ seen, float* __restrict__ theta) {
+    if (!*seen) return;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -489,24 +495,29 @@ cudaError_t launch_final_csr_gram(const int64_t* row_ptr, const int32_t* col, co
     double* Gp = P + d * d;
     float* MT = reinterpret_cast<float*>(Gp + gram_partial_doubles(k, d));
     float2* Pdf = reinterpret_cast<float2*>(reinterpret_cast<uintptr_t>(MT + k * d + 3) & ~uintptr_t(7));
+    int* seen = reinterpret_cast<int*>(Pdf + d * d);    // a row of more than 32 entries was met
+    cudaError_t e = cudaMemsetAsync(seen, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
     int tg = (int)((d * k + 255) / 256);
     if (tg > 152 * 8) tg = 152 * 8;
     k_transpose_mfull<<<tg, 256, 0, st>>>(Mfull, (int)d, (int)k, MT);
-    cudaError_t e = launch_gram_fp64(MT, d, k, d, Gp, P, status, st);           // P = Mfull Mfull^T (FP64-grade)
+    e = launch_gram_fp64(MT, d, k, d, Gp, P, status, st);           // P = Mfull Mfull^T (FP64-grade)
     if (e != cudaSuccess) return e;
     k_split_pairs<<<152 * 4, 256, 0, st>>>(P, d * d, Pdf);
     const bool vec = (reinterpret_cast<uintptr_t>(Mfull) % 16 == 0) && (k % 4 == 0);
     int64_t grid = (n + 255) / 256;                     // 32 rows a warp at a time
     if (grid > 152 * 24) grid = 152 * 24;
     if (grid < 1) grid = 1;
-    k_final_csr_pairs<<<(unsigned)grid, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Pdf, theta);  // empty rows too
+    k_final_csr_pairs<<<(unsigned)grid, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Pdf, seen, theta);  // empty rows too
     int64_t grid_l = (n + 255) / 256;                   // 32 rows scanned a warp
     if (grid_l > 152 * 16) grid_l = 152 * 16;
     if (grid_l < 1) grid_l = 1;
     if (vec)
-        k_final_csr_long<true><<<(unsigned)grid_l, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Mfull, (int)k, theta);
+        k_final_csr_long<true><<<(unsigned)grid_l, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Mfull, (int)k, seen,
+                                                                theta);
     else
-        k_final_csr_long<false><<<(unsigned)grid_l, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Mfull, (int)k, theta);
+        k_final_csr_long<false><<<(unsigned)grid_l, 256, 0, st>>>(row_ptr, col, val, n, (int)d, Mfull, (int)k, seen,
+                                                                 theta);
     return cudaGetLastError();
 }
 

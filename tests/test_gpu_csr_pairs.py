@@ -45,3 +45,33 @@ def test_pairs_at_the_edges_of_the_row_classes(length, d):
     assert np.all(np.abs(got - want) <= 2.0 ** -24 * np.abs(want) + 2.0 ** -38 * scale)
     assert L.lev_device_status(h) == 0
     h.close()
+
+
+@pytest.mark.parametrize("n", [31, 33, 1100, 40000])
+def test_long_rows_among_short_ones(n):
+    """Rows of more than 32 entries, whose pass runs only when the short rows' pass met one: every row gets its score
+    whichever group it is in, with one matrix after the other on the same handle."""
+    import torch
+    L = lev_module()
+    h = L.Handle(0)
+    d, k = 200, 512
+    rng = np.random.default_rng(n)
+    M = rng.standard_normal((d, k)).astype(np.float32)
+    M64 = M.astype(np.float64)
+    for frac in (0.2, 0.0, 0.2):
+        lens = np.where(rng.random(n) < frac, rng.integers(33, 80, n), rng.integers(0, 12, n))
+        if frac:
+            lens[-1] = 33
+        row_ptr, col, val = _rows(lens, d, rng, outside=False)
+        theta = torch.full((n,), -1.0, dtype=torch.float32, device="cuda")
+        L.lev_final_csr(h, to_dev(row_ptr), to_dev(col), to_dev(val), n, d, to_dev(M), "fp32", theta)
+        got = to_np(theta).astype(np.float64)
+        for i in list(range(min(n, 200))) + list(range(max(0, n - 200), n)):
+            e = slice(row_ptr[i], row_ptr[i + 1])
+            v = val[e].astype(np.float64)
+            want = float(((v @ M64[col[e]]) ** 2).sum())
+            # FP32 sums of at most 80 products a column, squared and summed over k: first-order bound
+            bound = float(((np.abs(v) @ np.abs(M64[col[e]])) ** 2).sum())
+            assert abs(got[i] - want) <= 2.0 ** -24 * (2 * 82 * bound + (k // 32 + 40) * want)
+        assert np.all(got >= 0)
+    h.close()
