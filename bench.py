@@ -429,11 +429,11 @@ def main():
                      f"permutation ({n} rows) and Omega ({d} x {cfg['k']}) for a new seed (lev_prepare)")
     # kernels of one lev_estimate_dense step with the bucket permutation, G and Omega cached:
     # CountSketch (FP32 B, or for the BF16 forms the Gaussian stage's operand itself), the Gaussian
-    # stage (split-K SGEMM or tcgen05 GEMM) and its reduction; Gram + reduce + the fill of the exchange
-    # rows + pivoted Cholesky + the FP64 conversion of R + two assembly kernels; the coefficient split
+    # stage (split-K SGEMM or tcgen05 GEMM) and its reduction; Gram + reduce + pivoted Cholesky (one
+    # cluster at d <= 256) + the FP64 conversion of R + two assembly kernels; the coefficient split
     # and the solve of the right factor; the final pass (tensor-core forms: plus its width and
     # operand packing kernels)
-    kernels_per_step = (3 + (1 if args.sketch_prec == "tf32" else 0) + 7 + 2
+    kernels_per_step = (3 + (1 if args.sketch_prec == "tf32" else 0) + 6 + 2
                         + (1 if args.final_prec == "fp32" else 3))
 
     rank_found = L.lev_estimate_dense(h, A, p, theta)          # also generates and caches G
@@ -594,7 +594,8 @@ def main():
         gram_ms.append(g_ms)
         chol_ms.append(f_ms)
     L.lev_set_timing(h, False)
-    pchol_name = "k_pchol_grid_reg"
+    # one thread-block cluster up to d = 256, a cooperative grid above
+    pchol_name = "k_pchol_cluster" if d <= 256 else "k_pchol_grid_reg"
     kernel_ms = {"k_final_tc": final_ms[args.final_prec], pchol_name: float(np.median(chol_ms)),
                  "k_gram_dot2+reduce": float(np.median(gram_ms))}
 
@@ -651,7 +652,7 @@ def main():
                          "pchol_us_per_step": kernel_ms[pchol_name] * 1e3 / max(1, r),
                          "householder_equivalent_fp64_flops": qf,
                          "note": f"{r} sequential pivot steps; one exchange of the pivot column per step "
-                                 "(through L2)"}
+                                 f"({'shared memory across the cluster' if d <= 256 else 'L2'})"}
     rooflines["pchol"] = {"kernel": pchol_name, "bound": "alu",
                           "achieved": chol_flops / (kernel_ms[pchol_name] * 1e-3) / 1e12, "peak": fp64_peak,
                           "unit": "TFLOP/s", "peak_source": "FP64 FMA rate measured on this GB300 (1.19 TFLOP/s)",
