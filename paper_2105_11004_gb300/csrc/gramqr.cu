@@ -616,7 +616,9 @@ __global__ void __launch_bounds__(kClRows * T, 1) k_pchol_cluster(const double* 
     __syncthreads();
     cl_sync();                                       // every CTA's F is filled before any is read
 
-    // the warp's largest active diagonal entry (key, lowest index among equal keys) into buffer b
+    // the warp's largest active diagonal entry (key, lowest index among equal keys) into buffer b. Searches
+    // alternate between the buffers (the first one takes 1, step j takes j mod 2): a warp may be a barrier behind,
+    // still reading the last search's
     auto warp_pick = [&](int b) {
         const unsigned long long k = active ? df_key(dg) : 0ull;
         const unsigned hi = (unsigned)(k >> 32), lo = (unsigned)k;
@@ -659,14 +661,14 @@ __global__ void __launch_bounds__(kClRows * T, 1) k_pchol_cluster(const double* 
         if (forced) {
             if (t == 0 && i == f0) s_next[0] = active ? dg : make_float2(0.f, 0.f);
         } else if (t == 0) {
-            warp_pick(0);
+            warp_pick(1);                             // step 0 writes buffer 0 with no barrier after these reads
         }
         __syncthreads();
         if (forced) {
             p = f0;
             sp = (p >= 0 && p < d) ? s_next[0] : make_float2(0.f, 0.f);
         } else {
-            p = block_pick(0, sp);
+            p = block_pick(1, sp);
         }
         go = p >= 0 && p < d && sp.x > 0.f && sp.x < 3.0e38f;
         if (go) thr = df_key(df_from_double(tau * tau * df_to_double(sp)));
@@ -832,7 +834,8 @@ __global__ void __launch_bounds__(NT, 1) k_pchol_grid_reg(const double* __restri
     bool active = row_ok;
 
     // the warp's largest active diagonal entry (key, lowest index among equals) into buffer b; after the barrier
-    // every warp combines the warps' results the same way
+    // every warp combines the warps' results the same way. Searches alternate between the buffers (the first one
+    // takes 1, step j takes j mod 2): a warp may be a barrier behind, still reading the last search's
     auto warp_pick = [&](int b) {
         const unsigned long long k = active ? df_key(dg) : 0ull;
         const unsigned hi = (unsigned)(k >> 32), lo = (unsigned)k;
@@ -884,14 +887,14 @@ __global__ void __launch_bounds__(NT, 1) k_pchol_grid_reg(const double* __restri
         if (forced) {
             if (i == f0) s_next[0] = dg;
         } else {
-            warp_pick(0);
+            warp_pick(1);                                  // step 0 writes buffer 0 with no barrier after these reads
         }
         __syncthreads();
         if (forced) {
             p = f0;
             sp = (p >= 0 && p < d) ? s_next[0] : make_float2(0.f, 0.f);
         } else {
-            p = block_pick(0, sp);
+            p = block_pick(1, sp);
         }
         go = p >= 0 && p < d && sp.x > 0.f && sp.x < 3.0e38f;
         if (go) thr = df_key(df_from_double(tau * tau * df_to_double(sp)));
