@@ -15,8 +15,11 @@
 //     of 2^(-8 i0 - 24), so digit i0 + 3 leaves nothing), so a row has at most four of these products, and over
 //     a chunk of 256 rows the sum stays inside 24 bits: the accumulators of g = 0 .. 6 are exact. Pairs with
 //     i + j > 6 are dropped (2^-56);
-//   * every 256 rows the accumulators join a running FP32 pair per entry of the tile, and the partial sums of
-//     the row splits are scaled back (powers of two) and added in FP64 in a fixed order.
+//   * every 256 rows the accumulators join a running FP32 pair per entry of the tile. The pair drifts with the
+//     length of its sum (each of a chunk's seven additions rounds at 2^-48 of it, the same way where rows repeat:
+//     constant columns were 4.8e-13 off after 341 chunks, 1.4e-11 after 9,766), so it joins an FP64 number every
+//     8 chunks; the partial sums of the row splits are scaled back (powers of two) and added in FP64 in a fixed
+//     order.
 // Measured against a 64-bit product, relative to sqrt(G_ii G_jj) and through the factor R^T R (whose own
 // rounding is about 5e-14): 7.2e-14 at 4096 x 1024 Gaussian (7.5e-14 with the compensated sums), 1.8e-14 with
 // rows scaled by e^(2 N) (8.4e-14), 1.7e-14 at 4096 x 500 with e^(4 N) (4.7e-14), 2.3e-14 with one row 1e4
@@ -72,7 +75,8 @@ constexpr int kRing = 3;                                   // half steps of a th
 constexpr int kSlotFloats = kHalf * kConvThreads;
 constexpr int kRingBytes = kRing * kSlotFloats * 4;
 constexpr int kMaxRows = 128;                               // rows of a block of column maxima
-constexpr int kUnitDoubles = kTile * kTile + kTile;        // a unit's partial tile (FP32 pairs) and 256 exponents
+constexpr int kFlush = 8;                                   // chunks after which a tile's pairs join FP64 numbers
+constexpr int kUnitDoubles = kTile * kTile + kTile;        // a unit's partial tile (FP64, or FP32 pairs) and 256 exponents
 constexpr uint64_t kWaitNs = 2000000000ull;
 constexpr int32_t kStatusGramTimeout = 5;
 
@@ -155,6 +159,7 @@ struct GramPlan {
     int nt, noff;              // 128-column blocks, tiles above the diagonal
     int splits, rows;          // row splits of every tile, rows a split
     int chunk;                 // rows a chunk (multiple of 16, at most kMaxChunk)
+    int flush;                 // kFlush where a split has more chunks (partial tiles in FP64), else 0 (FP32 pairs)
 };
 
 __device__ __forceinline__ void off_tile(int t, int nt, int& bi, int& bj) {
@@ -223,6 +228,15 @@ __global__ void __launch_bounds__(512) k_gram_colmax(const float* __restrict__ A
     __syncthreads();
     if (g == 0 && col < d)
         out[blockIdx.x * (int64_t)d + col] = max(max(part[0][c], part[1][c]), max(part[2][c], part[3][c]));
+}
+
+// x 2^k as a double, by its bits (FP64 conversions and multiplies run at 1/64 of the integer rate): x zero,
+// normal or not finite; -252 <= k <= 244.
+__device__ __forceinline__ double scaled_double(float x, int k) {
+    const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+    const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + ((uint32_t)(896 + k) << 20));
+    if (e == 0xffu) return __hiloint2double(0x7ff80000, 0);
+    return e == 0 ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
 }
 
 __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(const float* __restrict__ A, int64_t lda, int64_t m, int d,
@@ -424,67 +438,79 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(const float* __restrict
         asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
         const int lq = warp & 3, cg = warp >> 2;
         const uint32_t tacc = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(cg * 64);
-        f32x2 h[32], l[32];
+        double* out = unit + (cg * 64) * kTile + lq * 32 + lane;   // column-major (lanes write consecutive rows)
+        if (pl.flush)
+            for (int j = 0; j < 64; ++j) out[j * kTile] = 0.0;
+        int seg = 0;
+        do {                                               // the chunks of one running pair
+            f32x2 h[32], l[32];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) h[j] = l[j] = 0ull;
-        for (int seg = 0; seg < nseg; ++seg) {
-            // add the pass's accumulators: error-free for g <= 3; the sums of g >= 4 (about 2^-27 of the largest
-            // entry's square) join the low parts
-            const int pass = seg & 1;
-            wait_or_abort(smem_u32(&ctl->tfull), (uint32_t)(seg & 1), ctl, status);
-            __syncwarp();
-            tc_fence_after();
-            const int nacc = pass == 0 ? 4 : 3;
-            for (int a = 0; a < nacc; ++a) {
+            for (int j = 0; j < 32; ++j) h[j] = l[j] = 0ull;
+            const int end = pl.flush ? min(nseg, seg + 2 * kFlush) : nseg;
+            for (; seg < end; ++seg) {
+                // add the pass's accumulators: error-free for g <= 3; the sums of g >= 4 (about 2^-27 of the largest
+                // entry's square) join the low parts
+                const int pass = seg & 1;
+                wait_or_abort(smem_u32(&ctl->tfull), (uint32_t)(seg & 1), ctl, status);
+                __syncwarp();
+                tc_fence_after();
+                const int nacc = pass == 0 ? 4 : 3;
+                for (int a = 0; a < nacc; ++a) {
 #pragma unroll
-                for (int j0 = 0; j0 < 64; j0 += 8) {
-                    uint32_t r[8];
-                    tmem_ld8(tacc + (uint32_t)(a * kTile + j0), r);
-                    tmem_ld_wait();
-                    if (j0 == 56) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) {
-                            mbar_arrive(smem_u32(&ctl->afree[a]));
-                            if (pass == 1 && a == 2) mbar_arrive(smem_u32(&ctl->afree[3]));
+                    for (int j0 = 0; j0 < 64; j0 += 8) {
+                        uint32_t r[8];
+                        tmem_ld8(tacc + (uint32_t)(a * kTile + j0), r);
+                        tmem_ld_wait();
+                        if (j0 == 56) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) {
+                                mbar_arrive(smem_u32(&ctl->afree[a]));
+                                if (pass == 1 && a == 2) mbar_arrive(smem_u32(&ctl->afree[3]));
+                            }
+                        }
+                        if (pass == 0) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                f32x2& hj = h[j0 / 2 + j];
+                                const f32x2 v = pack2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+                                const f32x2 s1 = add2(hj, v), z = sub2(s1, hj);
+                                const f32x2 er = add2(sub2(hj, sub2(s1, z)), sub2(v, z));   // h + v = s1 + er
+                                hj = s1;
+                                l[j0 / 2 + j] = add2(l[j0 / 2 + j], er);
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                l[j0 / 2 + j] = add2(l[j0 / 2 + j], pack2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1])));
                         }
                     }
-                    if (pass == 0) {
+                }
+                if (pass == 1) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            f32x2& hj = h[j0 / 2 + j];
-                            const f32x2 v = pack2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
-                            const f32x2 s1 = add2(hj, v), z = sub2(s1, hj);
-                            const f32x2 er = add2(sub2(hj, sub2(s1, z)), sub2(v, z));   // h + v = s1 + er
-                            hj = s1;
-                            l[j0 / 2 + j] = add2(l[j0 / 2 + j], er);
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            l[j0 / 2 + j] = add2(l[j0 / 2 + j], pack2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1])));
+                    for (int j = 0; j < 32; ++j) {
+                        const f32x2 s1 = add2(h[j], l[j]), z = sub2(s1, h[j]);
+                        l[j] = add2(sub2(h[j], sub2(s1, z)), sub2(l[j], z));
+                        h[j] = s1;
                     }
                 }
             }
-            if (pass == 1) {
+            // the pairs as they are, or into the partial tile's FP64 numbers (this thread's alone: the additions
+            // in L2 come in its order, and nothing waits for them)
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const f32x2 s1 = add2(h[j], l[j]), z = sub2(s1, h[j]);
-                    l[j] = add2(sub2(h[j], sub2(s1, z)), sub2(l[j], z));
-                    h[j] = s1;
+            for (int j = 0; j < 32; ++j) {
+                float h0, h1, l0, l1;
+                unpack2(h[j], h0, h1);
+                unpack2(l[j], l0, l1);
+                if (pl.flush) {
+                    atomicAdd(out + 2 * j * kTile, scaled_double(h0, 0) + scaled_double(l0, 0));
+                    atomicAdd(out + (2 * j + 1) * kTile, scaled_double(h1, 0) + scaled_double(l1, 0));
+                } else {
+                    reinterpret_cast<float2*>(out)[2 * j * kTile] = make_float2(h0, l0);
+                    reinterpret_cast<float2*>(out)[(2 * j + 1) * kTile] = make_float2(h1, l1);
                 }
             }
-        }
-        // the partial tile as FP32 pairs, column-major (lanes write consecutive rows)
-        float2* out = reinterpret_cast<float2*>(unit) + lq * 32 + lane;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            float h0, h1, l0, l1;
-            unpack2(h[j], h0, h1);
-            unpack2(l[j], l0, l1);
-            out[(cg * 64 + 2 * j) * kTile] = make_float2(h0, l0);
-            out[(cg * 64 + 2 * j + 1) * kTile] = make_float2(h1, l1);
-        }
+        } while (seg < nseg);
     }
     tc_fence_before();
     __syncthreads();
@@ -494,15 +520,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(const float* __restrict
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }
-}
-
-// x 2^k as a double, by its bits (FP64 conversions and multiplies run at 1/64 of the integer rate): x zero,
-// normal or not finite; -252 <= k <= 244.
-__device__ __forceinline__ double scaled_double(float x, int k) {
-    const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
-    const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + ((uint32_t)(896 + k) << 20));
-    if (e == 0xffu) return __hiloint2double(0x7ff80000, 0);
-    return e == 0 ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
 }
 
 // G (d x d, both triangles) from the units' partials: scaled back and added in FP64. A CTA takes a 32 x 4
@@ -527,15 +544,18 @@ __global__ void __launch_bounds__(256) k_gram_tc_reduce(const double* __restrict
         const double* u = p + z * stride;
         const int32_t* ex = reinterpret_cast<const int32_t*>(u + T);
         const int er = ex[r0 + tx] - 14;
-        const float2* v = reinterpret_cast<const float2*>(u);
-        float2 x[4];
+        double x[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = v[(c0 + q) * kTile + r0 + tx];
+        for (int q = 0; q < 4; ++q) x[q] = u[(c0 + q) * kTile + r0 + tx];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int k = er + ex[kTile + c0 + q];
-            s[q] += scaled_double(x[q].x, k);
-            s[q] += scaled_double(x[q].y, k);
+            if (pl.flush) {
+                s[q] += x[q] * __hiloint2double((1023 + k) << 20, 0);
+            } else {                                        // the pair (high part in the low word)
+                s[q] += scaled_double(__int_as_float(__double2loint(x[q])), k);
+                s[q] += scaled_double(__int_as_float(__double2hiint(x[q])), k);
+            }
         }
     }
 #pragma unroll
@@ -596,6 +616,7 @@ GramPlan make_plan(int64_t m, int64_t d) {
     p.splits = (int)std::max<int64_t>(1, (m + p.rows - 1) / p.rows);
     const int n = (p.rows + kMaxChunk - 1) / kMaxChunk;
     p.chunk = std::min(kMaxChunk, ((p.rows + n - 1) / n + 15) / 16 * 16);
+    p.flush = (p.rows + p.chunk - 1) / p.chunk > kFlush ? kFlush : 0;
     return p;
 }
 
