@@ -11,10 +11,10 @@
 //    reduction of the split partials (tensor-core forms live in tc_sketch.cu).
 #include <cuda_bf16.h>
 
-#include <algorithm>
 #include <climits>
 
 #include "f32x2.cuh"
+#include "gauss_plan.cuh"
 #include "lev_common.cuh"
 #include "lev_kernels.cuh"
 
@@ -521,7 +521,8 @@ __global__ void __launch_bounds__(256) k_sgemm_splitk(
 
 // The same product with a 128 x 256 tile, 16 x 8 outputs per thread as packed row pairs (the loop of
 // k_final_dense_fp32: half the shared-memory reads a product of the 8 x 8 tile, which kept the FMA pipe at
-// 0.44), 16-byte loads: N > 128, K and N multiples of 4, 16-byte aligned operands. kchunk is a multiple of 16.
+// 0.44), 16-byte loads: K and N multiples of 4, 16-byte aligned operands (gauss_plan.cuh chooses). kchunk is a
+// multiple of 16.
 constexpr int SW_BM = 128, SW_BN = 256, SW_BK = 16;
 
 __global__ void __launch_bounds__(256, 1) k_sgemm_splitk_wide(
@@ -748,36 +749,19 @@ cudaError_t launch_gen_gaussian(int64_t m, int64_t s, int64_t ld, uint64_t seed,
     return cudaGetLastError();
 }
 
-static bool sgemm_wide(int64_t d, int64_t s) { return d > 128 && d % 4 == 0 && s % 4 == 0; }
-
-// Split-K of the FP32 stage: two waves of the wide tile (one CTA an SM) or about four 128 x 128 tiles an SM, which
-// is the same length of an FP32 chain; at least 256 k a split, 64 where that leaves SMs idle (m = 80, d = 20,
-// s = 1,600: 30 us on 7 CTAs).
-int gaussian_stage_splits(int64_t m, int64_t d, int64_t s) {
-    const bool wide = sgemm_wide(d, s);
-    const int64_t tiles = wide ? ((m + SW_BM - 1) / SW_BM) * ((d + SW_BN - 1) / SW_BN)
-                               : ((m + SG_BM - 1) / SG_BM) * ((d + SG_BN - 1) / SG_BN);
-    int64_t splits = wide ? std::max<int64_t>(1, 304 / tiles) : (608 + tiles - 1) / tiles;
-    const int64_t per = ((s + 255) / 256) * tiles >= 152 ? 256 : 64;
-    const int64_t max_by_k = (s + per - 1) / per;
-    if (splits > max_by_k) splits = max_by_k;
-    if (splits < 1) splits = 1;
-    return (int)splits;
-}
+int gaussian_stage_splits(int64_t m, int64_t d, int64_t s) { return (int)gauss_plan(m, d, s).splits; }
 
 cudaError_t launch_gaussian_stage_fp32(const float* G, const float* B, int64_t m, int64_t s,
                                        int64_t d, float* partial, int splits, float* Atilde,
                                        cudaStream_t st) {
-    int64_t kchunk = (s + splits - 1) / splits;
+    const GaussPlan p = gauss_plan(m, d, s);
     // G, B and the partials are buffers of the handle (256-byte aligned)
-    if (sgemm_wide(d, s)) {
-        kchunk = (kchunk + SW_BK - 1) / SW_BK * SW_BK;
+    if (p.wide) {
         dim3 grid((unsigned)((d + SW_BN - 1) / SW_BN), (unsigned)((m + SW_BM - 1) / SW_BM), (unsigned)splits);
-        k_sgemm_splitk_wide<<<grid, 256, 0, st>>>(G, B, (int)m, (int)d, s, kchunk, partial);
+        k_sgemm_splitk_wide<<<grid, 256, 0, st>>>(G, B, (int)m, (int)d, s, p.kchunk, partial);
     } else {
-        kchunk = (kchunk + SG_BK - 1) / SG_BK * SG_BK;
         dim3 grid((unsigned)((d + SG_BN - 1) / SG_BN), (unsigned)((m + SG_BM - 1) / SG_BM), (unsigned)splits);
-        k_sgemm_splitk<<<grid, 256, 0, st>>>(G, B, (int)m, (int)d, s, kchunk, partial);
+        k_sgemm_splitk<<<grid, 256, 0, st>>>(G, B, (int)m, (int)d, s, p.kchunk, partial);
     }
     k_reduce_splits<<<grid_for(m * d, 256, 152 * 8), 256, 0, st>>>(partial, splits, m * d, Atilde);
     return cudaGetLastError();
