@@ -41,7 +41,8 @@ int fail(int code, const char* fmt, ...) {
 // LEV_FAULT=timeout the read of the device status word after a synchronisation, and
 // LEV_FAULT=pivwait has the pivoted Cholesky withhold one published pivot column, so that the
 // bounded waits for it run out on the device (no trap, no fault: the kernels record the timeout in
-// the status word and return).
+// the status word and return). LEV_FAULT=partition has the pivoted Cholesky launch as on a part of a
+// GPU with 100 SMs and no room for a cluster.
 bool fault_is(const char* kind) {
     const char* f = getenv("LEV_FAULT");
     return f && strcmp(f, kind) == 0;
@@ -629,6 +630,7 @@ int handle_scratch(lev_handle* h, int which, size_t bytes, void** out) {
 }
 int handle_num_sms(lev_handle* h) { return h->num_sms; }
 bool fault_pivot_wait() { return fault_is("pivwait"); }
+bool fault_partition() { return fault_is("partition"); }
 const cudaEvent_t* handle_final_marks(lev_handle* h) {
     if (!h->timing) return nullptr;
     h->final_timed = true;

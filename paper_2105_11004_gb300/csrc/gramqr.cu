@@ -23,8 +23,8 @@
 //     gram_tc.cu takes its place (1.03 -> 0.18 ms at 4096 x 1024);
 //   k_pchol_cluster (d <= 256): one thread-block cluster of 8 or 16 CTAs, whose CTAs
 //     are scheduled together.
-//   k_pchol_grid_reg: one cooperative grid (two columns a CTA up to d = 256, at
-//     most one CTA per SM above); CTA c owns the columns l = c mod gridDim of the
+//   k_pchol_grid_reg (d > 256): one cooperative grid, at most one CTA per SM;
+//     CTA c owns the columns l = c mod gridDim of the
 //     Schur complement, row i of them in the registers of thread i, in
 //     double-float arithmetic (FP32 pairs, about 48 bits; FP64 runs at 1/64 of
 //     the FP32 rate here). All CTAs keep a replicated Schur diagonal and take the
@@ -33,8 +33,9 @@
 //     pivot publishes its updated column, unscaled, as soon as it is up to date,
 //     and the others wait for that row only (no flag, no grid barrier per step).
 //     The double-float helpers live in df.cuh;
-//   k_pchol_grid: the same with the columns in shared memory, for a GPU (or a
-//     partition of one) with fewer SMs than the register form's columns need.
+//   k_pchol_grid: the same with the columns in shared memory, for a partition of a
+//     GPU with fewer SMs than the register form's columns need or no room for a
+//     cluster.
 //
 // The Gram route resolves |R_jj| / |R_00| down to about sqrt(m u) ~ 1e-7; the
 // caller uses the Householder kernel when tau is below 1e-6 or d > 1024.
@@ -791,7 +792,7 @@ __device__ __forceinline__ f32x2 select2(bool c, f32x2 a, f32x2 b) {
 // row buffer alternates (one barrier a step instead of two) and every thread takes the next pivot and its inverse
 // root itself. Same exchange, arithmetic, outputs and stopping rule as k_pchol_grid; the pivots and R are the same.
 // Measured, us a step, columns in shared memory -> here: d = 1024 3.07 -> 2.35 (the updates of 32 warps bound it
-// here), d = 512 1.98 -> 1.38, d = 257 1.64 -> 1.44. Up to d = 256 it runs only where no cluster can be resident.
+// here), d = 512 1.98 -> 1.38, d = 257 1.64 -> 1.44.
 template <int NT, int COLS>
 __global__ void __launch_bounds__(NT, 1) k_pchol_grid_reg(const double* __restrict__ Gm, int d, int m, double tau,
                                                           const int32_t* __restrict__ forced, int forced_rank,
@@ -1178,7 +1179,8 @@ cudaError_t launch_pivoted_cholesky(int64_t m, int64_t d, double tau, const int3
     // cluster cannot be resident). Its CTAs are scheduled together, so factorisations of other streams never wait
     // on it half resident. The register grid below is faster alone (1.17 against 1.64 us a step at d = 256), but
     // with six batches in flight its 128-CTA grids held the SMs part by part until their bounded waits gave up.
-    if (d >= 1 && d <= 256) {
+    const bool partition = fault_partition();
+    if (d >= 1 && d <= 256 && !partition) {
         if (d <= 128)
             e = launch_pchol_cluster<16, 2>(8, m, d, tau, forced, forced_rank, q, status, st);
         else if ((e = launch_pchol_cluster<16, 2>(16, m, d, tau, forced, forced_rank, q, status, st)) ==
@@ -1187,26 +1189,24 @@ cudaError_t launch_pivoted_cholesky(int64_t m, int64_t d, double tau, const int3
         if (e != cudaErrorNotSupported) return e;
     }
     // Cooperative grid over the SMs, at most one CTA per SM; the grid does not change the result (every CTA takes
-    // the same pivots, each entry sees the same operations). One thread a row of S: 256, 512 or 1,024 threads. Up
-    // to d = 256 a CTA takes two columns (one packed pair): a step is latency and d / 2 CTAs are the shortest
-    // (d = 256: 1.24 us a step on 128 CTAs, 1.28 on 86, 1.26 on 64, 1.31 on 43, 1.33 on 32; whole estimates with
-    // other batches in flight are as fast or faster too). Above, all SMs: the updates count. The columns go to
-    // registers where they fit (128 SMs or more, any full GPU of this kind), else to shared memory.
+    // the same pivots, each entry sees the same operations). One thread a row of S: 256, 512 or 1,024 threads. Above
+    // d = 256 all SMs, as the updates count, and the columns go to registers where they fit (128 SMs or more, any
+    // full GPU of this kind). Fewer SMs, or no room for a cluster up to d = 256, where a step is latency and three
+    // columns a CTA leave SMs to other work: the columns in shared memory.
     int sms = 0, dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if (partition && sms > 100) sms = 100;
     if (sms < 1 || d < 1 || d > kGridMaxD) return cudaErrorInvalidValue;
     const int nt = d <= 256 ? 256 : d <= 512 ? 512 : 1024;
-    const int cols = nt / 128;
+    const int cols = d <= 256 ? 0 : nt / 128;             // columns a CTA of the register form
     int pgrid = sms < (int)d ? sms : (int)d;
-    if (d <= 256 && pgrid > (int)(d + 1) / 2) pgrid = (int)(d + 1) / 2;
+    if (d <= 256 && pgrid > (int)(d + 2) / 3) pgrid = (int)(d + 2) / 3;
     const size_t ncl = ((size_t)d + pgrid - 1) / pgrid;
     if (ncl > 32) return cudaErrorInvalidConfiguration;          // per-CTA bookkeeping holds 32 columns
     const bool reg = ncl <= (size_t)cols;
     const size_t smem = reg ? 0 : sizeof(float2) * (ncl * d + 3 * (size_t)d) + sizeof(int) * (size_t)d + 64;
-    const void* fn = reg ? nt == 256   ? (const void*)k_pchol_grid_reg<256, 2>
-                           : nt == 512 ? (const void*)k_pchol_grid_reg<512, 4>
-                                       : (const void*)k_pchol_grid_reg<1024, 8>
+    const void* fn = reg ? nt == 512 ? (const void*)k_pchol_grid_reg<512, 4> : (const void*)k_pchol_grid_reg<1024, 8>
                      : nt == 256 ? (const void*)k_pchol_grid<256>
                      : nt == 512 ? (const void*)k_pchol_grid<512>
                                  : (const void*)k_pchol_grid<1024>;
