@@ -21,8 +21,7 @@
 //     Upper 32 x 32 tiles split over rows, split partials reduced in a fixed
 //     order and mirrored. From 1.5e8 products on the tensor-core kernel of
 //     gram_tc.cu takes its place (1.03 -> 0.18 ms at 4096 x 1024);
-//   k_pchol_cluster (d <= 256): one thread-block cluster of 8 or 16 CTAs, whose CTAs
-//     are scheduled together.
+//   k_pchol_cluster (d <= 256): one thread-block cluster of 8 or 16 CTAs.
 //   k_pchol_grid_reg (d > 256): one cooperative grid, at most one CTA per SM;
 //     CTA c owns the columns l = c mod gridDim of the
 //     Schur complement, row i of them in the registers of thread i, in
@@ -1176,9 +1175,9 @@ cudaError_t launch_pivoted_cholesky(int64_t m, int64_t d, double tau, const int3
                                     const QrScratch& q, int32_t* status, cudaStream_t st) {
     cudaError_t e;
     // d <= 256: one cluster (16 columns a CTA: 8 CTAs up to d = 128, 16 above; 32 columns on 8 CTAs where a 16-CTA
-    // cluster cannot be resident). Its CTAs are scheduled together, so factorisations of other streams never wait
-    // on it half resident. The register grid below is faster alone (1.17 against 1.64 us a step at d = 256), but
-    // with six batches in flight its 128-CTA grids held the SMs part by part until their bounded waits gave up.
+    // cluster cannot be resident). It leaves the other SMs to the batches in flight: six estimates at once take
+    // 0.57 ms each at 1e6 x 256 and 0.13 at 20,000 x 256, 0.63 and 0.20 with the register grid below on 128 CTAs,
+    // which is the faster one alone (1.17 against 1.64 us a step at d = 256; the estimate 1.01 against 1.12 ms).
     const bool partition = fault_partition();
     if (d >= 1 && d <= 256 && !partition) {
         if (d <= 128)
