@@ -253,6 +253,13 @@ def run_reference(args, cfg):
     print(json.dumps(out), flush=True)
 
 
+def gram_kernels(m, d):
+    """Kernels that form the Gram matrix of an m x d FP32 matrix (the library's rule)."""
+    if d > 32 and m * d * (d + 32) >= 3.0e8:
+        return "k_gram_colmax + k_gram_tc + k_gram_tc_reduce"
+    return "k_gram_dot2 + k_gram_reduce"
+
+
 def qr_flops(m, d, r):
     """FP64 flops of the pivoted Householder QR that stops at rank r (norm recompute included)."""
     f = 0.0
@@ -596,8 +603,9 @@ def main():
     L.lev_set_timing(h, False)
     # one thread-block cluster up to d = 256, a cooperative grid above
     pchol_name = "k_pchol_cluster" if d <= 256 else "k_pchol_grid_reg"
+    gram_name = gram_kernels(cfg["m"], d)
     kernel_ms = {"k_final_tc": final_ms[args.final_prec], pchol_name: float(np.median(chol_ms)),
-                 "k_gram_dot2+reduce": float(np.median(gram_ms))}
+                 gram_name: float(np.median(gram_ms))}
 
     peaks, peak_src = load_peaks()
     hbm_peak = float(peaks["hbm_gbs"])
@@ -647,8 +655,8 @@ def main():
     qf = qr_flops(cfg["m"], d, r)
     fp64_peak = 1.19   # TFLOP/s, FP64 FMA rate measured on this GB300 (dependent-chain probe)
     chol_flops = 2.0 * sum((d - j) ** 2 for j in range(r))          # rank-1 updates of the trailing block
-    rooflines["rrqr"] = {"kernels": f"k_gram_dot2 + k_gram_reduce, {pchol_name}", "ms": stages["rrqr"],
-                         "gram_ms": kernel_ms["k_gram_dot2+reduce"], "pchol_ms": kernel_ms[pchol_name],
+    rooflines["rrqr"] = {"kernels": f"{gram_name}, {pchol_name}", "ms": stages["rrqr"],
+                         "gram_ms": kernel_ms[gram_name], "pchol_ms": kernel_ms[pchol_name],
                          "pchol_us_per_step": kernel_ms[pchol_name] * 1e3 / max(1, r),
                          "householder_equivalent_fp64_flops": qf,
                          "note": f"{r} sequential pivot steps; one exchange of the pivot column per step "
@@ -658,7 +666,8 @@ def main():
                           "unit": "TFLOP/s", "peak_source": "FP64 FMA rate measured on this GB300 (1.19 TFLOP/s)",
                           "algorithmic": chol_flops, "traffic": None, "ms": kernel_ms[pchol_name],
                           "note": "latency-bound: each pivot step waits for the pivot column from the CTA that "
-                                  "owns it (a round trip through L2) and a chain of dependent double-float "
+                                  f"owns it ({'a remote shared-memory hop' if d <= 256 else 'a round trip through L2'})"
+                                  " and a chain of dependent double-float "
                                   "(FP32 pair) operations; achieved is counted in FP64-equivalent flops, whose whole count "
                                   "would take ~9 us at the FP64 rate"}
     rooflines["pchol"]["frac"] = rooflines["pchol"]["achieved"] / fp64_peak
@@ -713,7 +722,7 @@ def main():
                         "rows_per_s": n / (ex_ms * 1e-3), "gram_ms": g_ms,
                         "gram_fp64_equivalent_tflops": 2.0 * gram_fma / (g_ms * 1e-3) / 1e12,
                         "fp64_peak_tflops": fp64_peak,
-                        "gram_note": "compensated FP32 sums (exact products, TwoSum blocks of 64 rows, FP64 outer sum)",
+                        "gram_note": gram_kernels(n, d),
                         "sketch_prec": args.sketch_prec, "final_prec": args.final_prec}
 
     # rank rules on the same batch's sketch (lev_rrqr_select): the diagonal test, the singular values
