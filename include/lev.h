@@ -120,7 +120,9 @@ int lev_destroy(lev_handle* h);
 const char* lev_last_error(void);
 
 /* Device memory the handle holds now, in bytes: its scratch buffers (grown on demand by the calls
- * made on it, never shrunk) and its caches of G, Omega and the CountSketch bucket permutation.
+ * made on it, never shrunk) and its caches of G, Omega and the CountSketch bucket permutation. The
+ * Gram matrix of an m x d matrix (the sketch's; A's in lev_exact_*) takes up to 4 MiB of partial sums
+ * below 1.5e8 products m d (d + 32) / 2, above up to 60 MB and m d / 32 bytes of column maxima.
  * Host only (no device work, no synchronisation). lev_destroy releases all of it.
  * Errors: LEV_EINVAL (NULL handle or bytes). */
 int lev_workspace_bytes(lev_handle* h, int64_t* bytes);

@@ -565,10 +565,11 @@ int check_csr(lev_handle* h, const int64_t* row_ptr, int64_t n, int64_t nnz, uin
 }
 
 // B = A^T A of CSR A (d x d FP64) as the sum of the rows' outer products (Lemma 8, Sec. 5.1): rows of
-// more than max(32, d / 5) entries are densified and their Gram formed by the compensated dense
-// kernel (about 30x the rate of the FP64 atomics per product, so it pays beyond about d / 5
-// entries); the others add their pairs by FP64 atomics. Synchronises `st` once (the count of long
-// rows sizes the dense part).
+// more than max(32, d / 5) entries are densified and their Gram formed by the dense kernels; the others
+// add their pairs by FP64 atomics. d / 5 is where the compensated dense kernel broke even (about 30x the
+// rate of the atomics per product). Many long rows now run on the tensor-core kernel at about six times
+// that rate, for which the line was not measured again. Synchronises `st` once (the count of long rows
+// sizes the dense part).
 int csr_gram(lev_handle* h, const int64_t* row_ptr, const int32_t* col, const float* val, int64_t n, int64_t d,
              double* G, cudaStream_t st) {
     const int64_t max_len = std::max<int64_t>(32, d / 5);

@@ -20,10 +20,11 @@
 //     constant columns were 4.8e-13 off after 341 chunks, 1.4e-11 after 9,766), so it joins an FP64 number every
 //     8 chunks; the partial sums of the row splits are scaled back (powers of two) and added in FP64 in a fixed
 //     order.
-// Measured against a 64-bit product, relative to sqrt(G_ii G_jj) and through the factor R^T R (whose own
-// rounding is about 5e-14): 7.2e-14 at 4096 x 1024 Gaussian (7.5e-14 with the compensated sums), 1.8e-14 with
-// rows scaled by e^(2 N) (8.4e-14), 1.7e-14 at 4096 x 500 with e^(4 N) (4.7e-14), 2.3e-14 with one row 1e4
-// times the others (1.6e-13).
+// Largest error of an entry against a 64-bit product, relative to sqrt(G_ii G_jj) (the compensated sums' in
+// brackets): 7.0e-15 at 4096 x 1024 Gaussian (1.1e-14), 2.0e-14 with rows scaled by e^(2 N) (9.7e-14); 1.7e-15 at
+// 1e6 x 256 Gaussian (5.1e-15), 4.5e-15 with rank 200 and e^(2 N) (1.1e-14), 1.5e-14 with e^(4 N) (8.9e-15); 3.3e-15
+// at 100,003 x 500 (4.6e-15), 3.2e-15 at 80,000 x 1,024 with a quarter of the entries (4.7e-15), 4.0e-14 at
+// 1e6 x 1,024 with constant columns (8.9e-13).
 //
 // Equal columns give bitwise equal rows and columns of G, as the symmetric compensated sums do (a pivot tie
 // goes to the lower index): the chunk sums are exact, and every tile has the same chunks and row splits, so
@@ -40,10 +41,10 @@
 //   * warp 16: allocates tensor memory and issues the MMAs (M = N = 128, K = 16);
 //   * warps 0..7 (fetchers): TMEM lane = row of the tile, 64 columns a warp; add a pass's accumulators to the
 //     running pairs and hand each accumulator back as soon as it is read.
-// The converters set the pace (two warps a scheduler; the MMAs are 48% of a tile's time above the diagonal):
-// 2.05 ms at 1e6 x 256, with the column maxima 0.17 ms and the sum of the splits 0.03 ms, against 17.1 ms for
-// the compensated sums; 0.15 + 0.03 ms
-// at 4096 x 1024 against 1.03 ms. Every wait is bounded; after a timeout the CTA runs on without waiting (its
+// The converters set the pace (two warps a scheduler; the tensor pipe is active 40% of the time at 4096 x 1024):
+// 2.19 ms at 1e6 x 256, with the column maxima 0.15 ms and the sum of the splits 0.02 ms, against 14.9 ms for
+// the compensated sums; 0.14 + 0.03 ms at 4096 x 1024 against 0.96 ms. The FP64 additions every 8 chunks cost less
+// than the runs differ (2.36 and 2.37 ms in all at 1e6 x 256, 2.63 and 2.64 at 80,000 x 1,024). Every wait is bounded; after a timeout the CTA runs on without waiting (its
 // barriers stay matched) and records the failure in the status word.
 #include <atomic>
 #include <cuda.h>
@@ -589,8 +590,8 @@ int device_sms() {
 // least 64 rows a split. In quarters of the time of a tile above the diagonal (0.124 us a row), one on the
 // diagonal takes three (0.094 us: its converters have half the work, the MMAs and fetches are the same), and
 // starting and ending a CTA about 260 rows. CTAs start in the order of their index, the long ones first. At
-// 1e6 x 256 that is 152 splits, every SM with one tile above and two on the diagonal (2.05 ms; 2.46 with 76
-// splits, 2.39 with 50 in one wave).
+// 1e6 x 256 that is 152 splits, every SM with one tile above and two on the diagonal (2.05 ms when the counts were
+// compared; 2.46 with 76 splits, 2.39 with 50 in one wave).
 GramPlan make_plan(int64_t m, int64_t d) {
     const int64_t sms = device_sms();
     GramPlan p;
