@@ -482,7 +482,9 @@ __global__ void k_scaled_transpose_df(const double* __restrict__ R, const int64_
 // With the factor Lc of Omega's Gram matrix (upper U, row q holding column q of L = U^T) and
 // r < k, r <= *d_kc, the right-hand side is column q of L_r instead and the columns q >= r stay 0.
 // us, with one CTA a column and a barrier a row before: d = k = 1,024 identity 1380 -> 375; d = 1,024,
-// k = 256 430 -> 228; r = 200, k = 256 41 -> 36.
+// k = 256 430 -> 228; r = 200, k = 256 41 -> 36. The first block takes no more rows than the last one with a
+// solution, in eights: of whole blocks r = 99, k = 150 took 29 us and r = 200, k = 256 (all 200 rows of Omega) 45,
+// more than before, now 25 and 40.
 constexpr int OMEGA_CH = 8, OMEGA_ST = 3;                     // rows a chunk, chunks in flight
 __global__ void __launch_bounds__(1024) k_omega_solve(const double* __restrict__ R, const float2* __restrict__ Rs,
                                                       const double* __restrict__ Om, const double* __restrict__ Lc,
@@ -513,12 +515,12 @@ __global__ void __launch_bounds__(1024) k_omega_solve(const double* __restrict__
     auto subtract = [&](float2 c, f32x2 bh, f32x2 bl) {
         df_sub_mul2(xh, xl, pack2(c.x, c.x), pack2(c.y, c.y), bh, bl);
     };
-    // The coefficients Rs[j][i] of this thread, j descending from the top block to its own, by chunks of 8
-    // rows through OMEGA_ST stages; 0 outside the strict triangle and past the rank. A thread reads only what
-    // it copied itself.
-    const int Jt = (identity ? q0 + ncol - 1 : r - 1) >> 5;
+    // The coefficients Rs[j][i] of this thread, j descending from the chunk of the last row with a solution that is
+    // not 0 to this warp's block, by chunks of 8 rows through OMEGA_ST stages; 0 outside the strict triangle and past
+    // the rank. A thread reads only what it copied itself.
+    const int last = identity ? q0 + ncol - 1 : r - 1, Jt = last >> 5;
     float2* ring = coefs + (size_t)w * (OMEGA_ST * OMEGA_CH * 32) + lane;
-    int next = Jt * 32 + 31, slot_in = 0, slot = 0;
+    int next = last | (OMEGA_CH - 1), slot_in = 0, slot = 0;
     auto copy_chunk = [&]() {
         if (next >= w * 32) {
             const unsigned to = (unsigned)__cvta_generic_to_shared(ring + slot_in * (OMEGA_CH * 32));
@@ -546,10 +548,11 @@ __global__ void __launch_bounds__(1024) k_omega_solve(const double* __restrict__
     for (int t = 0; t + 1 < OMEGA_ST; ++t) copy_chunk();
     for (int J = Jt; J >= 0; --J) {
         ulonglong2* buf = xs[J & 1];
+        const int top = J == Jt ? (last & 31) | (OMEGA_CH - 1) : 31;
         float2 c[OMEGA_CH];
         if (w == J) {
 #pragma unroll 1
-            for (int tb = 31; tb >= 0; tb -= OMEGA_CH) {
+            for (int tb = top; tb >= 0; tb -= OMEGA_CH) {
                 chunk(c);
 #pragma unroll
                 for (int u = 0; u < OMEGA_CH; ++u) {
@@ -563,7 +566,7 @@ __global__ void __launch_bounds__(1024) k_omega_solve(const double* __restrict__
         __syncthreads();
         if (w < J) {
 #pragma unroll 1
-            for (int tb = 31; tb >= 0; tb -= OMEGA_CH) {
+            for (int tb = top; tb >= 0; tb -= OMEGA_CH) {
                 chunk(c);
 #pragma unroll
                 for (int u = 0; u < OMEGA_CH; ++u) {
@@ -722,9 +725,11 @@ cudaError_t launch_omega_factor(const double* R, const int32_t* perm, const int6
         k_scaled_transpose_df<<<grid, 256, 0, st>>>(R, d_rank, (int)d, Rs2);
         const int threads = (int)((d + 31) / 32 * 32);
         const size_t smem = sizeof(float2) * (size_t)threads * OMEGA_CH * OMEGA_ST;
-        e = cudaFuncSetAttribute(k_omega_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(float2) * 1024 * OMEGA_CH * OMEGA_ST);
-        if (e != cudaSuccess) return e;
+        if (smem > 47 * 1024) {                                     // 1 KB more is static
+            e = cudaFuncSetAttribute(k_omega_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(float2) * 1024 * OMEGA_CH * OMEGA_ST);
+            if (e != cudaSuccess) return e;
+        }
         k_omega_solve<<<(unsigned)((k + 1) / 2), threads, smem, st>>>(R, Rs2, Omega, Lc && d_kc ? Lc : nullptr, (int)kc, d_kc,
                                                        perm, d_rank, (int)d, (int)k, omega_identity ? 1 : 0, Mfull);
         return cudaGetLastError();
