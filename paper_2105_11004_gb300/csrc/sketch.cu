@@ -300,8 +300,12 @@ __global__ void __launch_bounds__(256) k_countsketch_dense_scalar(
 // bounds meet there (44 warps an SM, with nearly no L1 left, took 11.5 ms).
 // A row costs four shuffles, and entries whose columns ascend strictly, as those
 // of sorted rows do, are added by plain loads and stores; other rows take
-// shared-memory atomics. 8e7 rows of 12 entries: 6.75 -> 6.38 ms; 2e6 of 8 and
-// 1% of 256: 253 -> 235 us.
+// shared-memory atomics. Among 32 rows with a longer one all entries stay in L1,
+// where a row's next sector often is, the next 32 entries are loaded while the
+// last are added, and all are atomics. The sketch (d = 1,024, split BF16) with all
+// entries kept in L1 and atomics, with all past L1 and the plain adds where they
+// may be, and as here: 2e6 rows of 8 entries 396, 379 and 366 us; 2e5 rows of 33
+// 128, 153 and 115; of 256 413, 426 and 354.
 constexpr int CS_PF = 8;
 __device__ __forceinline__ int32_t ld_entry(const int32_t* p) {
     int32_t v;
@@ -313,6 +317,66 @@ __device__ __forceinline__ float ld_entry(const float* p) {
     asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
+// The rows r0 .. of the warp's 32 (nr of them; lane r holds row r's bounds and length code), CS_PF at a time, into
+// sacc. LONG: some of the 32 have more than 32 entries.
+template <bool LONG>
+__device__ __forceinline__ void csr_rows_sum(const int32_t* __restrict__ col, const float* __restrict__ val, int d,
+                                             int64_t my_p0, int64_t my_p1, int my_len, int nr, int lane, float* sacc) {
+    for (int r0 = 0; r0 < nr; r0 += CS_PF) {
+        int cc[CS_PF], ln[CS_PF];
+        float vv[CS_PF];
+#pragma unroll
+        for (int u = 0; u < CS_PF; ++u) {                // loads of CS_PF rows in flight together
+            const int r = (r0 + u) & 31;                 // past nr: length 0
+            const int64_t p = __shfl_sync(0xffffffffu, my_p0, r) + lane;
+            ln[u] = __shfl_sync(0xffffffffu, my_len, r);
+            cc[u] = INT_MAX;
+            vv[u] = 0.f;
+            if (lane < (ln[u] & 63)) {
+                if (LONG) {
+                    cc[u] = __ldg(col + p);
+                    vv[u] = __ldg(val + p);
+                } else {
+                    cc[u] = ld_entry(col + p);
+                    vv[u] = ld_entry(val + p);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < CS_PF; ++u) {                // rows added in order
+            if (r0 + u >= nr) break;
+            const float sg = ln[u] & 64 ? -1.f : 1.f;
+            if (LONG) {
+                const bool more = (ln[u] & 63) > 32;
+                int64_t p = 0, p1 = 0;
+                int c2 = INT_MAX;
+                float v2 = 0.f;
+                if (more) {
+                    p1 = __shfl_sync(0xffffffffu, my_p1, r0 + u);
+                    p = __shfl_sync(0xffffffffu, my_p0, r0 + u) + 32 + lane;
+                    if (p < p1) { c2 = __ldg(col + p); v2 = __ldg(val + p); }
+                }
+                if ((unsigned)cc[u] < (unsigned)d) atomicAdd(&sacc[cc[u]], sg * vv[u]);
+                while (p < p1) {
+                    const int c = c2;
+                    const float v = v2;
+                    p += 32;
+                    if (p < p1) { c2 = __ldg(col + p); v2 = __ldg(val + p); }
+                    if ((unsigned)c < (unsigned)d) atomicAdd(&sacc[c], sg * v);
+                }
+            } else {
+                const int before = __shfl_up_sync(0xffffffffu, cc[u], 1);
+                const bool sorted = __all_sync(0xffffffffu, lane == 0 || before < cc[u] || cc[u] == INT_MAX);
+                if ((unsigned)cc[u] < (unsigned)d) {
+                    if (sorted) sacc[cc[u]] += sg * vv[u];
+                    else atomicAdd(&sacc[cc[u]], sg * vv[u]);
+                }
+            }
+            __syncwarp();
+        }
+    }
+}
+
 // Bucket b added into the warp's zeroed accumulator row sacc (d floats).
 __device__ __forceinline__ void csr_bucket_sum(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                                const float* __restrict__ val, int d, const int* __restrict__ off,
@@ -329,42 +393,8 @@ __device__ __forceinline__ void csr_bucket_sum(const int64_t* __restrict__ row_p
             my_p1 = row_ptr[row + 1];
             my_len = (int)max((int64_t)0, min((int64_t)33, my_p1 - my_p0)) + ((e & kSignBit) ? 64 : 0);
         }
-        for (int r0 = 0; r0 < nr; r0 += CS_PF) {
-            int cc[CS_PF], ln[CS_PF];
-            float vv[CS_PF];
-#pragma unroll
-            for (int u = 0; u < CS_PF; ++u) {                // loads of CS_PF rows in flight together
-                const int r = (r0 + u) & 31;                 // past nr: length 0
-                const int64_t p = __shfl_sync(0xffffffffu, my_p0, r) + lane;
-                ln[u] = __shfl_sync(0xffffffffu, my_len, r);
-                cc[u] = INT_MAX;
-                vv[u] = 0.f;
-                if (lane < (ln[u] & 63)) {
-                    cc[u] = ld_entry(col + p);
-                    vv[u] = ld_entry(val + p);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < CS_PF; ++u) {                // rows added in order
-                if (r0 + u >= nr) break;
-                const float sg = ln[u] & 64 ? -1.f : 1.f;
-                const int before = __shfl_up_sync(0xffffffffu, cc[u], 1);
-                const bool sorted = __all_sync(0xffffffffu, lane == 0 || before < cc[u] || cc[u] == INT_MAX);
-                if ((unsigned)cc[u] < (unsigned)d) {
-                    if (sorted) sacc[cc[u]] += sg * vv[u];
-                    else atomicAdd(&sacc[cc[u]], sg * vv[u]);
-                }
-                if ((ln[u] & 63) > 32) {
-                    __syncwarp();
-                    const int64_t p1 = __shfl_sync(0xffffffffu, my_p1, r0 + u);
-                    for (int64_t p = __shfl_sync(0xffffffffu, my_p0, r0 + u) + 32 + lane; p < p1; p += 32) {
-                        const int c = col[p];
-                        if ((unsigned)c < (unsigned)d) atomicAdd(&sacc[c], sg * val[p]);
-                    }
-                }
-                __syncwarp();
-            }
-        }
+        if (__any_sync(0xffffffffu, (my_len & 63) > 32)) csr_rows_sum<true>(col, val, d, my_p0, my_p1, my_len, nr, lane, sacc);
+        else csr_rows_sum<false>(col, val, d, my_p0, my_p1, my_len, nr, lane, sacc);
     }
 }
 
